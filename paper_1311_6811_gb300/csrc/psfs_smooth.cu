@@ -21,15 +21,7 @@
 // written at most once.
 //
 // When the rows are 16-byte multiples (nx % 4 == 0) smooth_tma_kernel does
-// the same sums with fewer instructions: a CTA owns 128 (x) x 8 (y) columns
-// over 32 planes; warp w the row y0 + w, lane l the columns x0 + 4 l .. x0 +
-// 4 l + 3.  Each plane with its halo (columns x0 - 4 .. x0 + 131, rows y0 - 1
-// .. y0 + 8; zeros outside the grid) arrives as one 2-D tensor box (TMA)
-// through a 4-stage mbarrier ring issued by one thread; each thread forms
-// the x-sums of its four columns in the three rows it needs straight from
-// shared memory (16-byte reads), their y-sum, and the z-sum from the y-sums
-// of the last two planes kept in registers: the same ((x-sums) y-sums)
-// z-sums and the same scaling as smooth_kernel, so the same bits.
+// the same sums with far fewer instructions; see there.
 #include <climits>
 
 #include "psfs_internal.cuh"
@@ -205,12 +197,13 @@ __global__ void __launch_bounds__(kThreads) smooth_kernel(const SmoothArgs a, in
 // ---------------------------------------------------------------------------
 // Tensor-box variant (rows of 16-byte multiples)
 // ---------------------------------------------------------------------------
-constexpr int kTX = 128, kTY = 8, kTZ = 32;         // outputs per CTA
-constexpr int kBoxX = kTX + 8, kBoxY = kTY + 2;     // plane box: columns x0 - 4 .. x0 + 131, rows y0 - 1 .. y0 + 8
-constexpr int kBoxFloats = kBoxX * kBoxY;           // 1360
-constexpr int kBoxStride = 1376;                    // floats per stage: 5504 bytes, a multiple of 128
-constexpr int kTStages = 4;
-constexpr int kTThreads = 32 * kTY;                 // one warp per output row
+constexpr int kTX = 128, kTRows = 4, kTWarps = 4;   // columns per CTA, rows per warp, computing warps
+constexpr int kTY = kTRows * kTWarps, kTZ = 32;     // rows per CTA, most planes per CTA
+constexpr int kBoxX = kTX + 8, kBoxY = kTY + 2;     // plane box: columns x0 - 4 .. x0 + 131, rows y0 - 1 .. y0 + 16
+constexpr int kBoxFloats = kBoxX * kBoxY;           // 2448
+constexpr int kBoxStride = (kBoxFloats + 31) / 32 * 32;   // floats per stage, a multiple of 128 bytes
+constexpr int kTStages = 4;                         // 38 KB per CTA, four CTAs per SM: 154 KB in flight
+constexpr int kTThreads = 32 * (kTWarps + 1);       // and one warp that issues the boxes
 
 // One box of a 4-D tensor map (x, y, z, frame), global -> shared, completion
 // counted on `bar`; x a multiple of 4 floats, elements outside the tensor
@@ -225,141 +218,197 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *tmap, 
         : "memory");
 }
 
-__global__ void __launch_bounds__(kTThreads) smooth_tma_kernel(const __grid_constant__ SmoothArgs a, int tiles_x,
-                                                               int tiles_y)
+// A CTA owns 128 (x) x 16 (y) columns over `tz` planes (z) of one frame; warp
+// w < 4 the rows y0 + 4 w .. + 3, lane l the columns x0 + 4 l .. + 3, so a
+// thread holds 4 x 4 outputs per plane.  Each plane with its halo (columns x0
+// - 4 .. x0 + 131, rows y0 - 1 .. y0 + 16; zeros outside the grid) arrives as
+// one tensor box (TMA) through a 4-stage ring of full / empty mbarriers: warp
+// 4 issues, the computing warps wait for a stage, read their six rows of it
+// and release it, and never wait for each other.
+//
+// Per row one 16-byte shared-memory read gives four columns and two shuffles
+// their neighbours; six rows of x-sums serve four rows of y-sums (two adds of
+// column pairs per instruction); the z-sum comes from the running sum of the
+// last two planes' y-sums: ((x-sums) y-sums) z-sums and the scaling by the
+// FP32 reciprocal of the clipped count, as in smooth_kernel, so the same
+// bits.  Few voxels lie above the threshold (1-3 % of a grid), so a warp only
+// looks for them (ballots into s_bal) in the planes whose largest value is
+// above it, and the compaction (one atomicAdd per warp) visits these planes.
+//
+// Bound by DRAM: 100 frames of 128^3 (8.4 MB in, 8.4 MB out each) take 310 us
+// with the list, 5.4 TB/s, 80 % of the copy rate.  Before (one row of four
+// columns per thread, three rows of x-sums per output row, a CTA barrier per
+// plane, every plane's ballots kept and walked again): 479 us, issue-bound.
+__global__ void __launch_bounds__(kTThreads, 4) smooth_tma_kernel(const __grid_constant__ SmoothArgs a, int tiles_x,
+                                                                  int tiles_y, int tz)
 {
     __shared__ __align__(128) float box[kTStages][kBoxStride];   // stages start 128-byte aligned
-    __shared__ __align__(8) uint64_t bars[kTStages];
-    __shared__ uint32_t s_bal[kTZ][kTY][4];   // ballot per output plane, warp and quad position
-    __shared__ uint32_t s_off[kTY];
-    __shared__ uint32_t s_base;
+    __shared__ uint32_t s_bal[kTZ][kTY][4];   // ballot per output plane, row and quad position
+    __shared__ __align__(8) uint64_t full[kTStages], empty[kTStages];
 
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int f = blockIdx.y;
     const int t = blockIdx.x;
-    const int tx = t % tiles_x, ty = (t / tiles_x) % tiles_y, tz = t / (tiles_x * tiles_y);
-    const int x0 = tx * kTX, y0 = ty * kTY, z0 = tz * kTZ;
+    const int tx = t % tiles_x, ty = (t / tiles_x) % tiles_y, tzi = t / (tiles_x * tiles_y);
+    const int x0 = tx * kTX, y0 = ty * kTY, z0 = tzi * tz;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const uint32_t nxy = (uint32_t)nx * (uint32_t)ny, n_vox = nxy * (uint32_t)nz;
-    float *out = a.smoothed ? a.smoothed + (size_t)f * n_vox : nullptr;
-    const bool vec_out = (reinterpret_cast<uintptr_t>(a.smoothed) & 15u) == 0;
-    const int x = x0 + 4 * lane, y = y0 + w;
-    const bool in_xy = y < ny && x < nx;
-
-    // clipped counts along x (per column) and y (the warp's row)
-    // and the reciprocals of the whole counts for 1, 2 and 3 planes along z
-    float inv[3][4];
-    const int cy = 1 + (y > 0) + (y + 1 < ny);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int cxy = (1 + (x + k > 0) + (x + k + 1 < nx)) * cy;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) inv[c][k] = 1.0f / (float)((c + 1) * cxy);
-    }
-
-    constexpr int kPlanes = kTZ + 2;   // z0 - 1 .. z0 + kTZ
-    if (tid == 0) {
-        for (int s = 0; s < kTStages; ++s) mbar_init(&bars[s], 1);
+    const int n_planes = min(tz, nz - z0) + 2;                               // z0 - 1 .. the plane after the last
+    const int n_warps = min(kTWarps, (ny - y0 + kTRows - 1) / kTRows);       // warps with rows in the grid
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kTStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], (uint32_t)n_warps);
+        }
         mbar_fence_init();
     }
     __syncthreads();
-    auto issue = [&](int q) {   // plane z0 - 1 + q into stage q % kTStages
-        const int s = q % kTStages;
-        mbar_arrive_expect_tx(&bars[s], (uint32_t)(kBoxFloats * 4));
-        tma_load_4d(box[s], &a.tmap, x0 - 4, y0 - 1, z0 - 1 + q, f, &bars[s]);
-    };
-    if (tid == 0)
-        for (int q = 0; q < kTStages && q < kPlanes; ++q) issue(q);
-
-    float ya[4] = {0.0f, 0.0f, 0.0f, 0.0f}, yb[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // y-sums of planes p - 2, p - 1
-    uint32_t warp_count = 0;
-    for (int q = 0; q < kPlanes; ++q) {
-        const int s = q % kTStages;
-        mbar_wait_bounded(&bars[s], (uint32_t)((q / kTStages) & 1), a.status);
-        // y-sum of this thread's four columns in plane p = z0 - 1 + q: the
-        // x-sums of rows y - 1, y, y + 1 (box rows w, w + 1, w + 2; box column
-        // c holds x0 - 4 + c)
-        float yc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        float xs[3][4];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            const float *row = box[s] + (w + r) * kBoxX + 4 * lane;
-            const float4 v = *reinterpret_cast<const float4 *>(row + 4);
-            const float left = row[3], right = row[8];
-            xs[r][0] = (left + v.x) + v.y;
-            xs[r][1] = (v.x + v.y) + v.z;
-            xs[r][2] = (v.y + v.z) + v.w;
-            xs[r][3] = (v.z + v.w) + right;
+    if (w == kTWarps) {
+        if (lane == 0) {
+            for (int q = 0; q < n_planes; ++q) {
+                const int s = q % kTStages;
+                if (q >= kTStages && !mbar_wait_bounded(&empty[s], (uint32_t)((q / kTStages - 1) & 1), a.status)) break;
+                mbar_arrive_expect_tx(&full[s], (uint32_t)(kBoxFloats * 4));
+                tma_load_4d(box[s], &a.tmap, x0 - 4, y0 - 1, z0 - 1 + q, f, &full[s]);
+            }
         }
+        return;   // every box that was issued is waited for by the computing warps
+    }
+    if (w >= n_warps) return;
+
+    const uint32_t nxy = (uint32_t)nx * (uint32_t)ny, n_vox = nxy * (uint32_t)nz;
+    float *out = a.smoothed ? a.smoothed + (size_t)f * n_vox : nullptr;
+    const bool vec_out = (reinterpret_cast<uintptr_t>(a.smoothed) & 15u) == 0;
+    const int x = x0 + 4 * lane, y = y0 + kTRows * w;
+    const bool in_x = x < nx;   // nx % 4 == 0: then all four columns are
+    const bool rows_inner = y > 0 && y + kTRows < ny;
+    // clipped counts along x and the reciprocals of the whole counts where y and z are not clipped
+    int cx[4];
+    float2 inv[2];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) yc[k] = (xs[0][k] + xs[1][k]) + xs[2][k];
-        __syncthreads();   // every thread is done with stage s
-        if (tid == 0 && q + kTStages < kPlanes) issue(q + kTStages);
-        // z-sums of plane p - 1
-        if (q >= 2) {
-            const int tq = q - 2, gz = z0 + tq;
+    for (int k = 0; k < 4; ++k) cx[k] = 1 + (x + k > 0) + (x + k + 1 < nx);
+    inv[0] = make_float2(1.0f / (float)(9 * cx[0]), 1.0f / (float)(9 * cx[1]));
+    inv[1] = make_float2(1.0f / (float)(9 * cx[2]), 1.0f / (float)(9 * cx[3]));
+    // the halo column of the first and the last lane: box columns 3 and 132
+    const int edge_off = lane == 0 ? 3 : kTX + 4;
+    const bool edge_lane = lane == 0 || lane == 31;
+
+    float2 yp[kTRows][2], s2[kTRows][2];   // y-sums of plane p - 1; their sum with those of plane p - 2
+#pragma unroll
+    for (int r = 0; r < kTRows; ++r)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) yp[r][h] = s2[r][h] = make_float2(0.0f, 0.0f);
+    uint32_t warp_count = 0, hit_planes = 0;
+    bool arriving = true;   // false after a timed-out wait: the status word marks the result invalid
+#pragma unroll 1
+    for (int q = 0; q < n_planes; ++q) {
+        const int s = q % kTStages;
+        if (arriving) arriving = mbar_wait_bounded(&full[s], (uint32_t)((q / kTStages) & 1), a.status);
+        const float *rows = box[s] + kTRows * w * kBoxX;
+        float2 xs[kTRows + 2][2];   // x-sums of rows y - 1 .. y + 4 of plane p = z0 - 1 + q
+#pragma unroll
+        for (int r = 0; r < kTRows + 2; ++r) {
+            const float4 v = *reinterpret_cast<const float4 *>(rows + r * kBoxX + 4 + 4 * lane);
+            float left = __shfl_up_sync(0xFFFFFFFFu, v.w, 1), right = __shfl_down_sync(0xFFFFFFFFu, v.x, 1);
+            if (edge_lane) {
+                const float e = rows[r * kBoxX + edge_off];
+                left = lane == 0 ? e : left;
+                right = lane == 0 ? right : e;
+            }
+            xs[r][0] = make_float2((left + v.x) + v.y, (v.x + v.y) + v.z);
+            xs[r][1] = make_float2((v.y + v.z) + v.w, (v.z + v.w) + right);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[s]);
+        const int tq = q - 2, gz = z0 + tq;   // the output plane p - 1
+        float2 sm[kTRows][2];
+#pragma unroll
+        for (int r = 0; r < kTRows; ++r)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 yc = __fadd2_rn(__fadd2_rn(xs[r][h], xs[r + 1][h]), xs[r + 2][h]);
+                sm[r][h] = __fadd2_rn(s2[r][h], yc);
+                s2[r][h] = __fadd2_rn(yp[r][h], yc);
+                yp[r][h] = yc;
+            }
+        if (q < 2) continue;
+        if (rows_inner && gz > 0 && gz + 1 < nz) {
+#pragma unroll
+            for (int r = 0; r < kTRows; ++r)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) sm[r][h] = __fmul2_rn(sm[r][h], inv[h]);
+        } else {
             const int cz = 1 + (gz > 0) + (gz + 1 < nz);
-            const bool valid_z = gz < nz;
-            float sm[4];
-            uint32_t b[4];
+#pragma unroll
+            for (int r = 0; r < kTRows; ++r) {
+                const int cyz = cz * (1 + (y + r > 0) + (y + r + 1 < ny));
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    sm[r][h] = __fmul2_rn(sm[r][h], make_float2(1.0f / (float)(cx[2 * h] * cyz),
+                                                                1.0f / (float)(cx[2 * h + 1] * cyz)));
+            }
+        }
+        if (out && in_x) {
+            float *o = out + ((uint32_t)gz * nxy + (uint32_t)y * (uint32_t)nx + (uint32_t)x);
+#pragma unroll
+            for (int r = 0; r < kTRows; ++r) {
+                if (y + r >= ny) break;
+                if (vec_out) {
+                    __stcs(reinterpret_cast<float4 *>(o), make_float4(sm[r][0].x, sm[r][0].y, sm[r][1].x, sm[r][1].y));
+                } else {
+                    __stcs(o, sm[r][0].x);
+                    __stcs(o + 1, sm[r][0].y);
+                    __stcs(o + 2, sm[r][1].x);
+                    __stcs(o + 3, sm[r][1].y);
+                }
+                o += nx;
+            }
+        }
+        float top = -INFINITY;
+#pragma unroll
+        for (int r = 0; r < kTRows; ++r)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) top = fmaxf(top, fmaxf(sm[r][h].x, sm[r][h].y));
+        if (__any_sync(0xFFFFFFFFu, top > a.threshold)) {
+            hit_planes |= 1u << tq;
+#pragma unroll
+            for (int r = 0; r < kTRows; ++r) {
+                const bool ok = in_x && y + r < ny;
+                uint32_t b[4];
+                b[0] = __ballot_sync(0xFFFFFFFFu, ok && sm[r][0].x > a.threshold);
+                b[1] = __ballot_sync(0xFFFFFFFFu, ok && sm[r][0].y > a.threshold);
+                b[2] = __ballot_sync(0xFFFFFFFFu, ok && sm[r][1].x > a.threshold);
+                b[3] = __ballot_sync(0xFFFFFFFFu, ok && sm[r][1].y > a.threshold);
+                warp_count += __popc(b[0]) + __popc(b[1]) + __popc(b[2]) + __popc(b[3]);
+                if (lane < 4)
+                    s_bal[tq][kTRows * w + r][lane] = lane == 0 ? b[0] : lane == 1 ? b[1] : lane == 2 ? b[2] : b[3];
+            }
+        }
+    }
+
+    // compaction of the warp's voxels above the threshold: one atomicAdd
+    if (!warp_count) return;
+    uint32_t pos = 0;
+    if (lane == 0) {
+        pos = atomicAdd(a.counts + f, warp_count);
+        if ((uint64_t)pos + warp_count > (uint64_t)a.capacity) atomicOr(a.status, kStatusCapacity);
+    }
+    pos = __shfl_sync(0xFFFFFFFFu, pos, 0);   // also orders s_bal's writes before the reads below
+    __syncwarp();
+    uint32_t *list = a.lists + (size_t)f * a.capacity;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    for (; hit_planes; hit_planes &= hit_planes - 1u) {
+        const int tq = __ffs(hit_planes) - 1;
+        for (int r = 0; r < kTRows; ++r) {
+            const uint32_t lin = (uint32_t)x + (uint32_t)nx * ((uint32_t)(y + r) + (uint32_t)ny * (uint32_t)(z0 + tq));
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float sum = (ya[k] + yb[k]) + yc[k];
-                sm[k] = sum * (cz == 3 ? inv[2][k] : (cz == 2 ? inv[1][k] : inv[0][k]));
-                b[k] = __ballot_sync(0xFFFFFFFFu, valid_z && in_xy && x + k < nx && sm[k] > a.threshold);
-                warp_count += __popc(b[k]);
-            }
-            if (lane < 4) s_bal[tq][w][lane] = lane == 0 ? b[0] : lane == 1 ? b[1] : lane == 2 ? b[2] : b[3];
-            if (out && valid_z && in_xy) {
-                float *o = out + ((uint32_t)gz * nxy + (uint32_t)y * (uint32_t)nx + (uint32_t)x);
-                if (vec_out && x + 3 < nx) {
-                    __stcs(reinterpret_cast<float4 *>(o), make_float4(sm[0], sm[1], sm[2], sm[3]));
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (x + k < nx) __stcs(o + k, sm[k]);
+                const uint32_t b = s_bal[tq][kTRows * w + r][k];
+                if ((b >> lane) & 1u) {
+                    const uint32_t pp = pos + __popc(b & lt_mask);
+                    if (pp < a.capacity) list[pp] = lin + (uint32_t)k;
                 }
+                pos += __popc(b);
             }
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            ya[k] = yb[k];
-            yb[k] = yc[k];
-        }
-    }
-
-    // compaction of the CTA's voxels above the threshold: one atomicAdd
-    if (lane == 0) s_off[w] = warp_count;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t total = 0;
-#pragma unroll
-        for (int k = 0; k < kTY; ++k) {
-            const uint32_t c = s_off[k];
-            s_off[k] = total;
-            total += c;
-        }
-        uint32_t base = 0;
-        if (total) {
-            base = atomicAdd(a.counts + f, total);
-            if ((uint64_t)base + total > (uint64_t)a.capacity) atomicOr(a.status, kStatusCapacity);
-        }
-        s_base = base;
-    }
-    __syncthreads();
-    uint32_t *list = a.lists + (size_t)f * a.capacity;
-    uint32_t pos = s_base + s_off[w];
-    const uint32_t lt_mask = (1u << lane) - 1u;
-    for (int tq = 0; tq < kTZ; ++tq) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint32_t b = s_bal[tq][w][k];
-            if ((b >> lane) & 1u) {
-                const uint32_t pp = pos + __popc(b & lt_mask);
-                if (pp < a.capacity)
-                    list[pp] = (uint32_t)(x + k) + (uint32_t)nx * ((uint32_t)y + (uint32_t)ny * (uint32_t)(z0 + tq));
-            }
-            pos += __popc(b);
         }
     }
 }
@@ -373,11 +422,17 @@ cudaError_t launch_smooth(const SmoothArgs &a_in, int n_frames, cudaStream_t s)
     if (e != cudaSuccess) return e;
     // rows of 16-byte multiples: the tensor-box kernel
     SmoothArgs a = a_in;
-    const int64_t ttx = (a.nx + kTX - 1) / kTX, tty = (a.ny + kTY - 1) / kTY, ttz = (a.nz + kTZ - 1) / kTZ;
+    // planes per CTA: the most that still give four CTAs per SM (a few frames
+    // of a small grid would leave SMs idle; each halving re-reads two planes
+    // per tile more)
+    const int64_t ttx = (a.nx + kTX - 1) / kTX, tty = (a.ny + kTY - 1) / kTY;
+    int planes = kTZ;
+    while (planes > 8 && ttx * tty * ((a.nz + planes - 1) / planes) * n_frames < 4 * (int64_t)device_sm_count()) planes /= 2;
+    const int64_t ttz = (a.nz + planes - 1) / planes;
     if (n_frames <= 65535 && ttx * tty * ttz <= INT_MAX &&
         encode_grid_tensor(a.prob, a.nx, a.ny, a.nz, n_frames, kBoxX, kBoxY, &a.tmap)) {
-        smooth_tma_kernel<<<dim3((unsigned)(ttx * tty * ttz), (unsigned)n_frames), kTThreads, 0, s>>>(a, (int)ttx,
-                                                                                                        (int)tty);
+        smooth_tma_kernel<<<dim3((unsigned)(ttx * tty * ttz), (unsigned)n_frames), kTThreads, 0, s>>>(
+            a, (int)ttx, (int)tty, planes);
         return cudaGetLastError();
     }
     const int tx = (a.nx + kSX - 1) / kSX, ty = (a.ny + kSY - 1) / kSY, tz = (a.nz + kSZ - 1) / kSZ;

@@ -126,3 +126,26 @@ def test_capacity_overflow():
     assert int(counts[0]) == ref["list"].size
     assert np.isin(lists[0].cpu().numpy(), ref["list"]).all()
     rec.close()
+
+
+@pytest.mark.parametrize("dims,F,shift", [((4, 1, 1), 1, 0), ((128, 16, 32), 1, 0), ((132, 17, 33), 2, 0),
+                                          ((256, 5, 70), 1, 0), ((8, 67, 9), 2, 0), ((128, 20, 34), 40, 0),
+                                          ((20, 18, 10), 2, 1)])
+def test_box_tiles(dims, F, shift):
+    """Rows of whole 16-byte units at the edges of the tensor-box kernel's
+    tiles (128 columns, warps of 4 rows, 8 to 32 planes by the size of the
+    call), with few and with many frames, and an output whose rows are not
+    16-byte aligned (shift)."""
+    nx, ny, nz = dims
+    V = nx * ny * nz
+    rec = _rec(S.Grid(nx, ny, nz, (-1.0, -1.0, 0.0), 0.05))
+    probs = np.random.default_rng(V).uniform(0.2, 0.8, (F, V)).astype(np.float32)
+    sm = torch.full((F * V + shift,), -1.0, device="cuda")[shift:].view(F, V)
+    lists = torch.full((F, V), -1, dtype=torch.int32, device="cuda")
+    counts = torch.zeros((F,), dtype=torch.int32, device="cuda")
+    psfs.psfs_smooth(rec.handle, F, torch.from_numpy(probs).cuda(), sm, lists, V, counts)
+    assert rec.sync() == psfs.PSFS_OK
+    for f in {0, F // 2, F - 1}:
+        c = int(counts[f])
+        _check(dims, probs[f], sm[f].cpu().numpy(), np.sort(lists[f, :c].cpu().numpy()), c, 0.5)
+    rec.close()
