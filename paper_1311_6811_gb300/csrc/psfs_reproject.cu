@@ -5,8 +5,16 @@
 // camera centre through the pixel centre meets, in front of the camera, the
 // cube of a listed voxel.
 //
-// One thread per (camera, listed voxel), with the forward kernels' matrices;
-// a CTA takes chunks of 256 consecutive listed voxels of one camera.  When
+// A CTA holds one camera's silhouette as a bitmask in shared memory (one bit
+// per pixel: 38 KB for 640 x 480), so every voxel of the frame's list sets its
+// pixels there, and the finished mask is written out once, as whole bytes,
+// zeros included: no memset before and no read-modify-write of the mask.
+// Images of more than kBandPixels take several CTAs, each a range of pixels;
+// when frames x cameras are few, a cluster of CTAs shares one mask, each with
+// every S-th chunk of the list, and each writes one part of the OR of the S
+// bitmasks, read through distributed shared memory.
+//
+// One thread per listed voxel, with the forward kernels' matrices.  When
 // all eight cube corners lie in front of the camera, a centre ray meets the
 // cube iff the pixel centre lies in the cube's projection: a convex polygon
 // whose vertices are the projections of the cube's silhouette loop (the
@@ -16,18 +24,14 @@
 // within or above each: 26 cases outside the cube), so a table made once on
 // the host gives the 4 or 6 corners to project.  A row of pixel centres
 // meets the polygon in one interval whose ends are the row's crossings with
-// its edges.  The chunk's intervals are set in shared memory when the union
-// of their boxes fits the stage, and each non-zero 4-byte word of the stage
-// is then OR-ed into the mask once; otherwise each interval is stored
-// directly (4-byte stores where whole aligned words are covered).  Cubes not
-// wholly in front of the camera, and projections too large for float32 rows,
-// take a float32 slab test of the centre ray of every pixel whose centre can
-// fall inside the projection's bounding box.  Every writer writes 1, so no
-// value is lost between writers.  Run on the surface list, the work is
-// proportional to the body's surface; the silhouette of a solid equals that
-// of its surface voxels.
+// its edges; the interval's bits are OR-ed into the words that lack them
+// (neighbouring surface voxels cover a pixel several times, so most words
+// need no atomic).  Cubes not wholly in front of the camera, and projections
+// too large for float32 rows, take a float32 slab test of the centre ray of
+// every pixel whose centre can fall inside the projection's bounding box.
+// Run on the surface list, the work is proportional to the body's surface;
+// the silhouette of a solid equals that of its surface voxels.
 #include <algorithm>
-#include <climits>
 #include <cmath>
 
 #include "psfs_internal.cuh"
@@ -36,7 +40,9 @@ namespace psfs {
 
 namespace {
 
-constexpr int kRpThreads = 256;
+constexpr int kRpThreads = 512;
+constexpr int kBandPixels = 98304 * 8;   // pixels of a CTA's bitmask: 96 KB, two CTAs per SM
+constexpr int kMaxCluster = 8;
 
 // Silhouette loops of a unit cube by camera region: entry (rx + 1) + 3 (ry +
 // 1) + 9 (rz + 1), r = -1 / 0 / +1 for a camera centre below / within /
@@ -102,18 +108,38 @@ SilTable make_sil_table()
     return t;
 }
 
-// Sets the pixels [x0, x1] of one mask row to 1: single bytes up to and after
-// the whole aligned 4-byte words in between (`words`: the row starts 4-byte
-// aligned), which get one 32-bit store each.
-__device__ __forceinline__ void set_run(uint8_t *row, int x0, int x1, bool words)
+// Sets the bits lo .. hi (lo <= hi) of a bitmask.  A word that already holds
+// them is only read: bits are never cleared, so a stale read costs an atomic,
+// not a bit.
+__device__ __forceinline__ void set_bits(uint32_t *bits, int lo, int hi)
 {
-    int x = x0;
-    if (words) {
-        for (; x <= x1 && (x & 3); ++x) row[x] = 1;
-        for (; x + 3 <= x1; x += 4) *reinterpret_cast<uint32_t *>(row + x) = 0x01010101u;
+    const int w0 = lo >> 5, w1 = hi >> 5;
+    for (int w = w0; w <= w1; ++w) {
+        uint32_t m = 0xFFFFFFFFu;
+        if (w == w0) m <<= lo & 31;
+        if (w == w1) m &= 0xFFFFFFFFu >> (31 - (hi & 31));
+        if (m & ~*reinterpret_cast<volatile uint32_t *>(bits + w)) atomicOr(bits + w, m);
     }
-    for (; x <= x1; ++x) row[x] = 1;
 }
+
+// Division by a run-time constant d: the estimate n floor(2^32 / d) / 2^32 is
+// at most one short.
+struct FastDiv {
+    uint32_t d, mul;   // mul = floor(2^32 / d), 2^32 - 1 for d = 1
+};
+
+__device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv &f, uint32_t &rem)
+{
+    uint32_t q = __umulhi(n, f.mul);
+    rem = n - q * f.d;
+    if (rem >= f.d) {
+        ++q;
+        rem -= f.d;
+    }
+    return q;
+}
+
+FastDiv make_fast_div(uint32_t d) { return {d, d == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d)}; }
 
 // The projection of one listed voxel's cube in camera c: the silhouette
 // polygon (n >= 3 corners, a 4-corner loop padded with its first corner, so
@@ -129,18 +155,26 @@ struct CubeProj {
     float o1[3];          // the cube's lower faces minus the camera centre (index coordinates)
 };
 
-__device__ __forceinline__ void project_cube(const ReprojectArgs &a, const SilTable &sil, int c, uint32_t v,
-                                             CubeProj &P)
+// `corners`: the silhouette table as corner offsets (see kernel).
+__device__ __forceinline__ void project_cube(const ReprojectArgs &a, const float4 *corners, const FastDiv &by_nxy,
+                                             const FastDiv &by_nx, int c, uint32_t v, CubeProj &P)
 {
-    const uint32_t nx = (uint32_t)a.nx, nxy = (uint32_t)a.nx * (uint32_t)a.ny;
-    const uint32_t kz = v / nxy, r = v - kz * nxy, jy = r / nx, ix = r - jy * nx;
+    uint32_t r, ix;
+    const uint32_t kz = fast_div(v, by_nxy, r), jy = fast_div(r, by_nx, ix);
     const int W = a.W, H = a.H;
     float m[12];
 #pragma unroll
     for (int q = 0; q < 12; ++q) m[q] = a.cam[c].m[q];
     // centred index coordinates of the cube's centre
     const float x0 = (float)ix - a.ci, y0 = (float)jy - a.cj, z0 = (float)kz - a.ck;
+    // all corners in front: depth of the centre beyond half the cube's extent
+    // in depth, with a margin far above the float32 rounding of a corner's
+    // depth; only cubes near the camera plane test their eight corners
+    const float w0 = fmaf(m[8], x0, fmaf(m[9], y0, fmaf(m[10], z0, m[11])));
+    const float ext = 0.5f * (fabsf(m[8]) + fabsf(m[9]) + fabsf(m[10]));
+    const float mag = fabsf(m[8] * x0) + fabsf(m[9] * y0) + fabsf(m[10] * z0) + fabsf(m[11]);
     bool behind = false;
+    if (!(w0 > 1.0001f * ext + 1e-5f * mag))
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const float X = x0 + ((q & 1) ? 0.5f : -0.5f), Y = y0 + ((q & 2) ? 0.5f : -0.5f),
@@ -161,14 +195,13 @@ __device__ __forceinline__ void project_cube(const ReprojectArgs &a, const SilTa
 #pragma unroll
     for (int ax = 2; ax >= 0; --ax)
         code = 3 * code + (P.o1[ax] > 0.0f ? 0 : (P.o1[ax] + 1.0f < 0.0f ? 2 : 1));
-    const uint32_t ent = sil.e[code];
-    const int n = (int)(ent & 15u);
+    const float4 *loop = corners + 6 * code;
+    const int n = (int)loop[0].w;
     float umin = INFINITY, umax = -INFINITY, vmin = INFINITY, vmax = -INFINITY;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        const int q = (int)((ent >> (4 + 3 * (k < n ? k : 0))) & 7u);
-        const float X = x0 + ((q & 1) ? 0.5f : -0.5f), Y = y0 + ((q & 2) ? 0.5f : -0.5f),
-                    Z = z0 + ((q & 4) ? 0.5f : -0.5f);
+        const float4 q = loop[k];
+        const float X = x0 + q.x, Y = y0 + q.y, Z = z0 + q.z;
         const float u = fmaf(m[0], X, fmaf(m[1], Y, fmaf(m[2], Z, m[3])));
         const float vv = fmaf(m[4], X, fmaf(m[5], Y, fmaf(m[6], Z, m[7])));
         // hardware reciprocal (about 1 ulp): the corners move by ~1e-7 of their
@@ -231,17 +264,19 @@ __device__ __forceinline__ void polygon_row(const CubeProj &P, int y, int &xs, i
 }
 
 // Slab test of the centre rays of the box's pixels (cubes not wholly in
-// front of the camera, or projections too large for float32 rows), stored
-// straight to the mask.
-__device__ void slab_test_pixels(const ReprojectArgs &a, int c, const CubeProj &P, uint8_t *mask)
+// front of the camera, or projections too large for float32 rows) within the
+// pixels p0 .. p1 - 1 of the band.
+__device__ void slab_test_pixels(const ReprojectArgs &a, int c, const CubeProj &P, uint32_t *bits, int p0, int p1)
 {
     float mi[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) mi[q] = a.inv[c].minv[q];
     const float o2[3] = {P.o1[0] + 1.0f, P.o1[1] + 1.0f, P.o1[2] + 1.0f};
-    for (int y = P.ya; y <= P.yb; ++y) {
+    const int yb = min(P.yb, (p1 - 1) / a.W);
+    for (int y = max(P.ya, p0 / a.W); y <= yb; ++y) {
         const float py = (float)y + 0.5f;
-        for (int x = P.xa; x <= P.xb; ++x) {
+        const int xb = min(P.xb, p1 - 1 - y * a.W);
+        for (int x = max(P.xa, p0 - y * a.W); x <= xb; ++x) {
             const float px = (float)x + 0.5f;
             float t_in = 0.0f, t_out = INFINITY;
 #pragma unroll
@@ -255,125 +290,172 @@ __device__ void slab_test_pixels(const ReprojectArgs &a, int c, const CubeProj &
                 t_in = fmaxf(t_in, fminf(t1, t2));
                 t_out = fminf(t_out, fmaxf(t1, t2));
             }
-            if (t_in <= t_out) mask[(size_t)y * a.W + x] = 1;
+            if (t_in <= t_out) set_bits(bits, y * a.W + x - p0, y * a.W + x - p0);
         }
     }
 }
 
-constexpr int kStageBytes = 32768;   // a CTA's staged mask region
-
-// A CTA takes chunks of kRpThreads consecutive listed voxels of one camera
-// (neighbours in space: the fusion compacts tile by tile), one voxel per
-// thread.  When the union of the chunk's polygon boxes fits kStageBytes
-// (rows of whole aligned 4-byte words), the chunk's rows are set in shared
-// memory and each non-zero word of the region is OR-ed into the mask once
-// (one atomicOr per word instead of a store per row run and voxel: the
-// projections of neighbouring surface voxels overlap several times);
-// otherwise each thread stores its runs directly.
-__global__ void __launch_bounds__(kRpThreads, 4) reproject_kernel(const __grid_constant__ ReprojectArgs a,
-                                                                  const __grid_constant__ SilTable sil)
+// ---- the cluster's other bitmasks (distributed shared memory) ----
+__device__ __forceinline__ uint32_t cluster_rank()
 {
-    __shared__ __align__(16) uint32_t stage[kStageBytes / 4];
-    __shared__ int s_box[4];   // -xa, xb, -ya, yb of the chunk
-    const int f = blockIdx.y;
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+__device__ __forceinline__ uint32_t load_peer(const uint32_t *p, uint32_t rank)
+{
+    uint32_t a, v;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// Word w of the OR of the S bitmasks.
+__device__ __forceinline__ uint32_t or_word(const uint32_t *bits, int w, int S)
+{
+    if (S == 1) return bits[w];
+    uint32_t v = 0;
+    for (int r = 0; r < S; ++r) v |= load_peer(bits + w, (uint32_t)r);
+    return v;
+}
+
+// The low four bits of v as four bytes of 0 or 1.
+__device__ __forceinline__ uint32_t spread4(uint32_t v) { return ((v & 15u) * 0x00204081u) & 0x01010101u; }
+
+// blockIdx.x = ((camera * bands) + band) * S + rank, blockIdx.y = frame.  The
+// pixels of a camera are numbered row by row; band b holds b * band_pix ..
+// min(W H, (b + 1) band_pix) - 1.
+//
+// Bound by issue (about 800 instructions per voxel and camera, most of them
+// the six edge tests of each pixel row): 100 frames of 4.7 K surface voxels, 8
+// cameras of 640 x 480, take 164 us.  Before (chunks of 256 voxels staged as
+// bytes over their common box, OR-ed into a zeroed mask word by word): 275 us;
+// with eight corner depths, corner offsets from selects and integer divisions
+// per voxel instead of the depth bound, the offset table and fast_div: 175 us.
+__global__ void __launch_bounds__(kRpThreads, 2) reproject_kernel(const __grid_constant__ ReprojectArgs a,
+                                                                  const __grid_constant__ SilTable sil,
+                                                                  FastDiv by_nxy, FastDiv by_nx, int bands,
+                                                                  int band_pix, int S)
+{
+    extern __shared__ __align__(16) uint32_t bits[];   // band_pix / 32 words and a zero word
+    // per camera region the corners of the silhouette loop as offsets from the
+    // cube's centre (.w: their number; a 4-corner loop padded with its first)
+    __shared__ float4 s_corners[27 * 6];
+    const int tid = threadIdx.x;
+    if (tid < 27 * 6) {
+        const uint32_t ent = sil.e[tid / 6], n = ent & 15u, k = tid % 6;
+        const uint32_t q = (ent >> (4 + 3 * (k < n ? k : 0))) & 7u;
+        s_corners[tid] = make_float4((q & 1) ? 0.5f : -0.5f, (q & 2) ? 0.5f : -0.5f, (q & 4) ? 0.5f : -0.5f, (float)n);
+    }
+    const int rank = S == 1 ? 0 : (int)cluster_rank();
+    const int cb = (int)blockIdx.x / S;
+    const int c = cb / bands, f = blockIdx.y;
+    const int K = a.n_cams, W = a.W, n_pix = a.W * a.H;
+    const int p0 = (cb - c * bands) * band_pix, p1 = min(n_pix, p0 + band_pix);
+    const int n_words = (p1 - p0 + 31) / 32 + 1;
+    for (int w = tid; w < n_words; w += kRpThreads) bits[w] = 0u;
+    __syncthreads();
+
     const uint32_t m_cnt = min(__ldg(a.counts + f), a.list_stride);
     const uint32_t *list = a.lists + (size_t)f * a.list_stride;
-    const int K = a.n_cams, W = a.W, H = a.H;
-    uint8_t *masks = a.masks + (size_t)f * K * W * H;
-    const bool words = (W % 4 == 0) && ((reinterpret_cast<uintptr_t>(a.masks) & 3u) == 0);
-    const uint32_t per_cam = (m_cnt + kRpThreads - 1) / kRpThreads;
-    const uint64_t n_chunks = (uint64_t)per_cam * K;
-    const int tid = threadIdx.x;
-    for (uint64_t ch = blockIdx.x; ch < n_chunks; ch += gridDim.x) {
-        const int c = (int)(ch / per_cam);
-        const uint32_t e = (uint32_t)(ch - (uint64_t)c * per_cam) * kRpThreads + tid;
-        uint8_t *mask = masks + (size_t)c * W * H;
+    const int y_lo = p0 / W, y_hi = (p1 - 1) / W;
+    for (uint64_t e = (uint64_t)rank * kRpThreads + tid; e < m_cnt; e += (uint64_t)S * kRpThreads) {
+        const uint32_t v = __ldg(list + e);
+        if (v >= a.n_vox) continue;
         CubeProj P;
-        P.n = 0;
-        bool have = false;
-        if (e < m_cnt) {
-            const uint32_t v = __ldg(list + e);
-            if (v < a.n_vox) {
-                project_cube(a, sil, c, v, P);
-                have = true;
-            }
-        }
-        const bool poly = have && P.n >= 3 && P.xa <= P.xb && P.ya <= P.yb;
-        // the chunk's box over its polygons (integer atomics in shared memory)
-        if (tid == 0) {
-            s_box[0] = s_box[1] = s_box[2] = s_box[3] = INT_MIN;
-        }
-        __syncthreads();
-        if (poly) {
-            atomicMax(&s_box[0], -P.xa);
-            atomicMax(&s_box[1], P.xb);
-            atomicMax(&s_box[2], -P.ya);
-            atomicMax(&s_box[3], P.yb);
-        }
-        __syncthreads();
-        int X0 = 0, Y0 = 0, rw = 0, rh = 0;
-        bool staged = false;
-        if (words && s_box[1] != INT_MIN) {
-            X0 = (-s_box[0]) & ~3;
-            const int X1 = s_box[1] | 3;   // W % 4 == 0: still inside the row
-            Y0 = -s_box[2];
-            rw = X1 - X0 + 1;
-            rh = s_box[3] - Y0 + 1;
-            staged = (int64_t)rw * rh <= kStageBytes;
-        }
-        if (staged) {
-            const int n_words = rw * rh / 4;
-            for (int w = tid; w < n_words; w += kRpThreads) stage[w] = 0u;
-            __syncthreads();
-            if (poly) {
-                uint8_t *st = reinterpret_cast<uint8_t *>(stage);
-                for (int y = P.ya; y <= P.yb; ++y) {
-                    int xs, xe;
-                    polygon_row(P, y, xs, xe);
-                    if (xs > xe ||
-                        !PSFS_IN_BOUNDS(y >= Y0 && y - Y0 < rh && xs >= X0 && xe - X0 < rw, a.status))
-                        continue;
-                    uint8_t *row = st + (y - Y0) * rw - X0;
-                    for (int x = xs; x <= xe; ++x) row[x] = 1;
-                }
-            }
-            __syncthreads();
-            const int row_words = rw / 4;
-            for (int w = tid; w < n_words; w += kRpThreads) {
-                const uint32_t val = stage[w];
-                if (val) {
-                    const int yy = w / row_words, xx = X0 + 4 * (w - yy * row_words);
-                    atomicOr(reinterpret_cast<unsigned int *>(mask + (size_t)(Y0 + yy) * W + xx), val);
-                }
-            }
-        } else if (poly) {
-            for (int y = P.ya; y <= P.yb; ++y) {
+        project_cube(a, s_corners, by_nxy, by_nx, c, v, P);
+        if (P.n >= 3) {
+            if (P.xa > P.xb) continue;
+            const int ye = min(P.yb, y_hi);
+            for (int y = max(P.ya, y_lo); y <= ye; ++y) {
                 int xs, xe;
                 polygon_row(P, y, xs, xe);
-                if (xs <= xe && PSFS_IN_BOUNDS(y >= 0 && y < H && xs >= 0 && xe < W, a.status))
-                    set_run(mask + (size_t)y * W, xs, xe, words);
+                if (xs > xe || !PSFS_IN_BOUNDS(y >= 0 && y < a.H && xs >= 0 && xe < W, a.status)) continue;
+                const int lo = max(y * W + xs, p0), hi = min(y * W + xe, p1 - 1);
+                if (lo <= hi) set_bits(bits, lo - p0, hi - p0);
             }
+        } else {
+            slab_test_pixels(a, c, P, bits, p0, p1);
         }
-        if (have && P.n < 3) slab_test_pixels(a, c, P, mask);
-        __syncthreads();   // the stage and the box are reused by the next chunk
     }
+    if (S == 1)
+        __syncthreads();
+    else
+        cluster_sync();
+
+    // this CTA's part of the band, bits as bytes: single bytes up to the
+    // first and after the last whole aligned 16 bytes
+    const int part = ((p1 - p0 + S - 1) / S + 31) & ~31;
+    const int q0 = p0 + rank * part, q1 = min(p1, q0 + part);
+    uint8_t *mask = a.masks + ((size_t)f * K + c) * n_pix;
+    if (q0 < q1) {
+        const int head = min(q1 - q0, (int)((16u - (uint32_t)(reinterpret_cast<uintptr_t>(mask + q0) & 15u)) & 15u));
+        const int n16 = (q1 - q0 - head) / 16, tail0 = q0 + head + 16 * n16;
+        for (int u = tid; u < n16; u += kRpThreads) {
+            const int b = q0 + head + 16 * u - p0, w = b >> 5, sh = b & 31;
+            uint32_t v = or_word(bits, w, S) >> sh;
+            if (sh > 16) v |= or_word(bits, w + 1, S) << (32 - sh);
+            *reinterpret_cast<uint4 *>(mask + p0 + b) =
+                make_uint4(spread4(v), spread4(v >> 4), spread4(v >> 8), spread4(v >> 12));
+        }
+        if (tid < 32) {
+            const int p = tid < 16 ? q0 + tid : tail0 + tid - 16;
+            if (tid < 16 ? tid < head : p < q1)
+                mask[p] = (uint8_t)((or_word(bits, (p - p0) >> 5, S) >> ((p - p0) & 31)) & 1u);
+        }
+    }
+    if (S > 1) cluster_sync();   // the peers read this CTA's bitmask until here
 }
 
 }  // namespace
 
+// Bands: as few as hold kBandPixels each (two CTAs per SM).  Cluster size: 1,
+// 2, 4 or 8 CTAs per mask, the smallest that gives four CTAs per SM in all, so
+// that a few frames still fill the GPU (9 frames of 5 cameras, 470 x 351: 24 us
+// with 8, 27 us with the chunked kernel before) and many frames write each mask
+// from one bitmask, without reading peers.
 cudaError_t launch_reproject(const ReprojectArgs &a, int n_frames, cudaStream_t s)
 {
     if (n_frames <= 0) return cudaSuccess;
     static const SilTable sil = make_sil_table();
-    cudaError_t e = cudaMemsetAsync(a.masks, 0, (size_t)n_frames * a.n_cams * a.W * a.H, s);
-    if (e != cudaSuccess) return e;
-    const int sms = device_sm_count();
-    // CTAs per frame: about 4 per SM over all frames, at most one per chunk
-    const uint64_t max_chunks = (uint64_t)((a.list_stride + kRpThreads - 1) / kRpThreads) * a.n_cams;
-    const uint32_t want = (uint32_t)std::max(1, 4 * std::max(sms, 1) / n_frames);
-    const uint32_t per_frame = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, max_chunks));
-    reproject_kernel<<<dim3(per_frame, (unsigned)n_frames), kRpThreads, 0, s>>>(a, sil);
-    return cudaGetLastError();
+    const int n_pix = a.W * a.H;
+    const int bands = (n_pix + kBandPixels - 1) / kBandPixels;
+    const int band_pix = ((n_pix + bands - 1) / bands + 31) & ~31;
+    const int smem = (band_pix / 32 + 1) * 4;
+    const int64_t masks = (int64_t)n_frames * a.n_cams * bands, want = 4 * (int64_t)std::max(device_sm_count(), 1);
+    int S = 1;
+    while (S < kMaxCluster && masks * S < want) S *= 2;
+    static bool configured[64] = {false};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!configured[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(reproject_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kBandPixels / 8 + 4);
+        if (e != cudaSuccess) return e;
+        configured[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.n_cams * bands * S), (unsigned)n_frames);
+    cfg.blockDim = dim3(kRpThreads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)S;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, reproject_kernel, a, sil, make_fast_div((uint32_t)a.nx * (uint32_t)a.ny),
+                                       make_fast_div((uint32_t)a.nx), bands, band_pix, S);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 }  // namespace psfs

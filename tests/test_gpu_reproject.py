@@ -135,3 +135,21 @@ def test_staged_and_direct_paths(width, height, n_set):
         _check(sc.grid, sc.cams, s_.astype(np.uint32), got[f])
         assert got[f].sum() > 100
     rec.close()
+
+
+@pytest.mark.parametrize("width,height,n_cams,frames", [(67, 51, 2, 1), (33, 1, 1, 3), (1100, 760, 1, 1),
+                                                        (67, 51, 3, 250)])
+def test_bitmask_bands_and_clusters(width, height, n_cams, frames):
+    """Masks whose bytes do not start 16-byte aligned (odd sizes), an image of
+    more pixels than one CTA's bitmask holds (two bands), one mask shared by a
+    cluster (few frames) and one CTA per mask (many frames)."""
+    sc = S.make_scene(seed=44, grid_n=20, cube_side=2.0, n_cams=n_cams, width=width, height=height,
+                      focal=0.9 * width)
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+    s_ = np.random.default_rng(5).choice(sc.grid.n_voxels, 60, replace=False).astype(np.int32)
+    lists = torch.from_numpy(s_).cuda().repeat(frames, 1)
+    counts = torch.full((frames,), s_.size, dtype=torch.int32, device="cuda")
+    got = _gpu_masks(rec, lists, counts, s_.size)
+    _check(sc.grid, sc.cams, s_.astype(np.uint32), got[0])
+    assert (got == got[0]).all()
+    rec.close()
