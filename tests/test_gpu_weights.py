@@ -114,3 +114,20 @@ def test_chain_from_images_ranks_the_true_pose_first():
     _check(sc.cams, m, parts, w, t)
     assert w[0] >= np.sort(w)[-3]   # the true pose among the best three of 30
     rec.close()
+
+
+@pytest.mark.parametrize("n_cams,n_parts,n_cyl,kt,kw", [(1, 1, 10, 8, 4), (7, 3, 10, 1, 1), (3, 5, 1, 64, 3),
+                                                        (5, 2, 9, 5, 64), (2, 1500, 10, 4, 2)])
+def test_clusters_and_sample_grids(n_cams, n_parts, n_cyl, kt, kw):
+    """One to eight CTAs per particle (by particles and cameras, cameras not a
+    multiple of them), sample grids of one and of the most samples per axis,
+    sample counts that are not whole warps."""
+    sc = S.make_scene(seed=53, grid_n=16, cube_side=2.2, n_cams=n_cams, width=101, height=77, focal=90.0)
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+    caps = S.body_capsules(S.random_pose(np.random.default_rng(11)), np.zeros((10, 3)))
+    masks = np.stack([(S.render_labels(c, caps) >= 0).astype(np.uint8) for c in sc.cams])
+    parts = _particles(12, n_parts, _cyl(caps))[:, :n_cyl]
+    w, t = _gpu(rec, parts, masks, kt, kw)
+    keep = np.unique(np.linspace(0, n_parts - 1, 8).astype(int))
+    _check(sc.cams, masks, parts[keep], w[keep], t[keep], kt, kw)
+    rec.close()
