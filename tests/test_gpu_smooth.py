@@ -149,3 +149,28 @@ def test_box_tiles(dims, F, shift):
         c = int(counts[f])
         _check(dims, probs[f], sm[f].cpu().numpy(), np.sort(lists[f, :c].cpu().numpy()), c, 0.5)
     rec.close()
+
+
+@pytest.mark.parametrize("dims,F,in_shift", [((1, 1, 1), 1, 0), ((129, 17, 9), 1, 0), ((131, 16, 33), 3, 0),
+                                             ((258, 5, 11), 1, 0), ((127, 33, 8), 2, 0), ((93, 20, 34), 30, 0),
+                                             ((93, 20, 34), 2, 1), ((64, 20, 10), 2, 1)])
+def test_rows_of_any_length(dims, F, in_shift):
+    """Rows that are not whole 16-byte units (row copies that start and end
+    inside one, voxel totals that do not fill the last one), tiles with a
+    neighbour column on either side, and grids that do not start 16-byte
+    aligned (in_shift)."""
+    nx, ny, nz = dims
+    V = nx * ny * nz
+    rec = _rec(S.Grid(nx, ny, nz, (-1.0, -1.0, 0.0), 0.05))
+    probs = np.random.default_rng(V).uniform(0.2, 0.8, (F, V)).astype(np.float32)
+    occ = torch.full((F * V + in_shift,), 9.0, device="cuda")
+    occ[in_shift:] = torch.from_numpy(probs).cuda().view(-1)
+    sm = torch.full((F, V), -1.0, device="cuda")
+    lists = torch.full((F, V), -1, dtype=torch.int32, device="cuda")
+    counts = torch.zeros((F,), dtype=torch.int32, device="cuda")
+    psfs.psfs_smooth(rec.handle, F, occ[in_shift:], sm, lists, V, counts)
+    assert rec.sync() == psfs.PSFS_OK
+    for f in {0, F // 2, F - 1}:
+        c = int(counts[f])
+        _check(dims, probs[f], sm[f].cpu().numpy(), np.sort(lists[f, :c].cpu().numpy()), c, 0.5)
+    rec.close()
