@@ -14,7 +14,9 @@
 //          segment (a two-level block scan);
 //   fill   the same projection again; each voxel claims a slot of its
 //          pixel's segment (integer atomics, so the order is arbitrary);
-//   sort   one thread per pixel sorts its segment by voxel index.
+//   sort   one warp per slice of 32 consecutive pixels sorts each pixel's
+//          segment by voxel index and lays the slice out for the pixel pass
+//          (see kSliceMax).
 //
 // The pixel pass of every frame then owns one pixel per thread and adds the
 // dLoss/dL of its segment's voxels in ascending voxel order: no float
@@ -22,6 +24,8 @@
 // or eight frames per pass), so the gradients are deterministic and the
 // batched pass is bit-identical to one frame per call.  The work is one load
 // per (voxel, camera) pair, instead of a walk along each pixel's ray.
+#include <algorithm>
+
 #include "psfs_fuse_common.cuh"
 
 namespace psfs {
@@ -80,24 +84,92 @@ __global__ void __launch_bounds__(256) owner_fill_kernel(const __grid_constant__
     }
 }
 
-// Insertion sort of each pixel's segment (segments hold a few voxels, the
-// voxels along the pixel's ray; this runs once per handle).
-__global__ void __launch_bounds__(256) owner_sort_kernel(const uint32_t *off, uint32_t *vox, int64_t n_pix)
+// Layout of the lists.  A slice is 32 consecutive pixels, one lane of a warp
+// each; its entries lie at vox[off[32 s] .. off[32 s + 32)).  In a slice of at
+// most kSliceMax entries they are jagged rows: first the first voxel of every
+// pixel that has one, in lane order, then the second voxels, and so on.  The
+// lanes of a warp that walk their lists together then read consecutive
+// entries: one or two lines per step, where a pixel's entries side by side
+// spread a step over eleven lines (11 voxels per pixel on average), which
+// took as many L1 wavefronts as the gathers they serve.  Nothing is padded.
+// Larger slices (more than 128 voxels per pixel: images much coarser than the
+// grid) keep each pixel's entries side by side at vox[off[p] .. off[p + 1]).
+constexpr uint32_t kSliceMax = 4096;
+constexpr int kSortWarps = 2;   // 32 KB of shared memory per CTA
+
+// Insertion sort of each pixel's segment by voxel index, one warp per slice
+// (in shared memory when the slice fits), then the jagged layout; once per
+// handle.
+__global__ void __launch_bounds__(32 * kSortWarps) owner_sort_kernel(const uint32_t *off, uint32_t *vox, int64_t n_pix)
 {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_pix; p += stride) {
-        const uint32_t e0 = off[p], e1 = off[p + 1];
-        for (uint32_t e = e0 + 1; e < e1; ++e) {
-            const uint32_t x = vox[e];
+    __shared__ uint32_t s_seg[kSortWarps][kSliceMax];
+    const int lane = threadIdx.x & 31;
+    uint32_t *buf = s_seg[threadIdx.x >> 5];
+    const int64_t n_slices = (n_pix + 31) / 32, stride = (int64_t)gridDim.x * kSortWarps;
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    for (int64_t sl = (int64_t)blockIdx.x * kSortWarps + (threadIdx.x >> 5); sl < n_slices; sl += stride) {
+        const uint32_t e0 = off[min(32 * sl + lane, n_pix)], e1 = off[min(32 * sl + lane + 1, n_pix)];
+        const uint32_t base = __shfl_sync(0xFFFFFFFFu, e0, 0), end = __shfl_sync(0xFFFFFFFFu, e1, 31);
+        const bool jagged = end - base <= kSliceMax;
+        uint32_t *seg = vox + base;
+        if (jagged) {
+            for (uint32_t e = lane; e < end - base; e += 32) buf[e] = seg[e];
+            __syncwarp();
+            seg = buf;
+        }
+        const uint32_t b0 = e0 - base, n = e1 - e0;
+        for (uint32_t e = b0 + 1; e < b0 + n; ++e) {
+            const uint32_t x = seg[e];
             uint32_t q = e;
-            while (q > e0 && vox[q - 1] > x) {
-                vox[q] = vox[q - 1];
+            while (q > b0 && seg[q - 1] > x) {
+                seg[q] = seg[q - 1];
                 --q;
             }
-            vox[q] = x;
+            seg[q] = x;
+        }
+        __syncwarp();
+        if (jagged) {
+            uint32_t pos = base;
+            for (uint32_t j = 0; __any_sync(0xFFFFFFFFu, j < n); ++j) {
+                const uint32_t has = __ballot_sync(0xFFFFFFFFu, j < n);
+                if (j < n) vox[pos + __popc(has & lt_mask)] = buf[b0 + j];
+                pos += __popc(has);
+            }
+            __syncwarp();   // the buffer is reused by the next slice
         }
     }
 }
+
+// One lane's walk along its pixel's list, K voxels per step, in ascending
+// voxel order; every lane of the warp walks with it (step needs them all).
+template <int K>
+struct OwnerWalk {
+    const uint32_t *next;   // jagged: the warp's next row; otherwise the lane's next entry
+    uint32_t left;          // entries of the lane not yet fetched
+    bool jagged;
+
+    // The slice's segment offsets: e0, e1 of this lane's pixel, the slice's ends.
+    __device__ __forceinline__ void init(const uint32_t *vox, uint32_t e0, uint32_t e1)
+    {
+        const uint32_t base = __shfl_sync(0xFFFFFFFFu, e0, 0), end = __shfl_sync(0xFFFFFFFFu, e1, 31);
+        jagged = end - base <= kSliceMax;
+        next = vox + (jagged ? base : e0);
+        left = e1 - e0;
+    }
+    // The next K voxels: v[k] for the first min(K, left) of them.
+    __device__ __forceinline__ void step(uint32_t (&v)[K])
+    {
+        const uint32_t lt_mask = (1u << (threadIdx.x & 31)) - 1u;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const bool has = (uint32_t)k < left;
+            const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, has);
+            v[k] = has ? __ldg(next + (jagged ? __popc(lanes & lt_mask) : 0)) : 0u;
+            next += jagged ? __popc(lanes) : 1;
+        }
+        left = left > (uint32_t)K ? left - (uint32_t)K : 0u;
+    }
+};
 
 // Exclusive scan of one block's kScanThreads values in registers.
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t *s_warp, uint32_t *total)
@@ -182,7 +254,7 @@ __global__ void __launch_bounds__(256) scan_add_kernel(uint32_t *out, int64_t n,
 //   dLoss/ds = acc (da / a(s) - db / b(s))            (Eq. 5-9, a, b linear in s)
 //   dLoss/dr = dLoss/ds s (1 - s), with s (1 - s) = u / (1 + u)^2 (no cancellation)
 //   dLoss/dmu_c, dLoss/dvar_c from dLoss/dr (Eq. 1).
-__device__ __forceinline__ void chain_rule_pre(const BackwardArgs &b, const uint8_t *im, const float (&mu)[3],
+__device__ __forceinline__ void chain_rule_pre(const BackwardArgs &b, const float (&im)[3], const float (&mu)[3],
                                                const float (&hh)[3], float base, float acc, float &dslm,
                                                float (&dm)[3], float (&dv)[3])
 {
@@ -192,9 +264,8 @@ __device__ __forceinline__ void chain_rule_pre(const BackwardArgs &b, const uint
     if (acc != 0.0f) {
         float dd[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) dd[c] = (float)im[c] - mu[c];
-        const float r = base + pixel_quad((float)im[0], (float)im[1], (float)im[2], mu[0], mu[1], mu[2], hh[0],
-                                          hh[1], hh[2]);
+        for (int c = 0; c < 3; ++c) dd[c] = im[c] - mu[c];
+        const float r = base + pixel_quad(im[0], im[1], im[2], mu[0], mu[1], mu[2], hh[0], hh[1], hh[2]);
         const float u = exp_fast(-fabsf(r));
         const float inv = rcp_approx(1.0f + u);
         const float s_val = r > 0.0f ? inv : u * inv;
@@ -218,48 +289,77 @@ __device__ __forceinline__ float chain_rule_slm(const BackwardArgs &b, int64_t p
     return acc * (div_fast(b.da, av) - div_fast(b.db, bv));
 }
 
-// One frame: pixel p sums b.dl over its segment in ascending voxel order.
+// An owner's index names a voxel of the grid (tested in the bounds-checked
+// build only).
+__device__ __forceinline__ bool owner_in_grid(const BackwardArgs &b, uint32_t v)
+{
+    (void)b;
+    (void)v;
+    return PSFS_IN_BOUNDS(v < (uint64_t)b.f.nx * b.f.ny * b.f.nz, b.f.status);
+}
+
+// The warps of the one-frame pixel pass take the slices of eight rows column
+// by column (about W / 32 slices make a row): the eight warps of a CTA then
+// work on eight rows of the same 32 columns, whose owners lie close together,
+// so that more of the 32-byte sectors their dL share (eight voxels along x)
+// are still in L1: 63.6 -> 59.6 us per 128^3 x 8 frame.  A permutation of the
+// slices, padded to whole groups of eight rows.  The group pass reads whole
+// 32-byte records, which no two owners share, and is faster in plain order
+// (218 against 238 us per 16 frames).
+__device__ __forceinline__ int64_t slice_of(int64_t i, uint32_t per_row)
+{
+    const int64_t rows = i / (8 * (int64_t)per_row);
+    const uint32_t in = (uint32_t)(i - rows * 8 * per_row);
+    return (rows * 8 + (in & 7u)) * per_row + (in >> 3);
+}
+
+// One frame: pixel p sums b.dl over its list in ascending voxel order, one
+// warp per slice.  Four owners' dL are in flight while the next four indices
+// load; the adds stay in ascending order.  Bound by the scattered dL reads, a
+// 32-byte sector for most owners: 59.6 us per 128^3 x 8 x 640 x 480 frame
+// (16.0 M owners), 67.8 before with each pixel's indices side by side.
 __global__ void __launch_bounds__(256) owner_pixel_kernel(const __grid_constant__ BackwardArgs b, const uint32_t *off,
                                                           const uint32_t *vox)
 {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < b.n_pix; p += stride) {
-        const uint32_t e0 = __ldg(off + p);
-        uint32_t e1 = __ldg(off + p + 1);
-#ifdef PSFS_BOUNDS_CHECK
-        {   // the pixel's segment lies in the lists and names voxels of the grid
-            const uint64_t n_vox = (uint64_t)b.f.nx * b.f.ny * b.f.nz;
-            bool seg_ok = PSFS_IN_BOUNDS(e0 <= e1 && e1 <= __ldg(off + b.n_pix), b.f.status);
-            for (uint32_t e = e0; seg_ok && e < e1; ++e) seg_ok = PSFS_IN_BOUNDS(__ldg(vox + e) < n_vox, b.f.status);
-            if (!seg_ok) e1 = e0;
-        }
-#endif
+    const uint32_t per_row = max(b.f.W / 32, 1);
+    const int64_t n_slices = (b.n_pix + 31) / 32, n_padded = (n_slices + 8 * per_row - 1) / (8 * per_row) * (8 * per_row);
+    const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
+    for (int64_t i = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; i < n_padded; i += stride) {
+        const int64_t sl = slice_of(i, per_row);
+        if (sl >= n_slices) continue;
+        const int64_t p = 32 * sl + (threadIdx.x & 31);
+        const uint32_t e0 = __ldg(off + min(p, b.n_pix)), e1 = __ldg(off + min(p + 1, b.n_pix));
+        OwnerWalk<4> walk;
+        walk.init(vox, e0, e1);
         float acc = 0.0f;
-        // four owners at a time: their index and dL loads are independent,
-        // so they are in flight together; the adds stay in ascending order
-        uint32_t e = e0;
-        for (; e + 4 <= e1; e += 4) {
-            const uint32_t v0 = __ldg(vox + e), v1 = __ldg(vox + e + 1), v2 = __ldg(vox + e + 2),
-                           v3 = __ldg(vox + e + 3);
-            const float d0 = __ldg(b.dl + v0), d1 = __ldg(b.dl + v1), d2 = __ldg(b.dl + v2), d3 = __ldg(b.dl + v3);
-            acc += d0;
-            acc += d1;
-            acc += d2;
-            acc += d3;
+        uint32_t v[4];
+        const uint32_t cnt = e1 - e0;
+        const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, cnt);
+        walk.step(v);
+        for (uint32_t j = 0; j < longest; j += 4) {
+            float d[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                d[k] = j + k < cnt && owner_in_grid(b, v[k]) ? __ldg(b.dl + v[k]) : 0.0f;
+            walk.step(v);
+            // a lane past its list adds +0, which leaves its sum (never -0) as it is
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc += d[k];
         }
-        for (; e < e1; ++e) acc += __ldg(b.dl + __ldg(vox + e));
+        if (p >= b.n_pix) continue;
         float dslm, dm[3], dv[3];
         if (b.img) {
-            float mu[3] = {0.0f, 0.0f, 0.0f}, hh[3] = {0.0f, 0.0f, 0.0f}, base = 0.0f;
+            float mu[3] = {0.0f, 0.0f, 0.0f}, hh[3] = {0.0f, 0.0f, 0.0f}, im[3] = {0.0f, 0.0f, 0.0f}, base = 0.0f;
             if (acc != 0.0f) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
+                    im[c] = (float)__ldg(b.img + 3 * p + c);
                     mu[c] = __ldg(b.mean + 3 * p + c);
                     hh[c] = __ldg(b.hinv + 3 * p + c);
                 }
                 base = pixel_log_base(hh[0], hh[1], hh[2], b.c0);
             }
-            chain_rule_pre(b, b.img + 3 * p, mu, hh, base, acc, dslm, dm, dv);
+            chain_rule_pre(b, im, mu, hh, base, acc, dslm, dm, dv);
         } else {
             dslm = chain_rule_slm(b, p, acc);
 #pragma unroll
@@ -274,34 +374,15 @@ __global__ void __launch_bounds__(256) owner_pixel_kernel(const __grid_constant_
 }
 
 // One voxel's 32-byte record of dLoss/dL (kBwRecord frames) with one 256-bit
-// read-only load.
-__device__ __forceinline__ void load_record(const float *rec, uint32_t (&w)[8])
+// read-only load; zeros, and no load, unless `on`.
+__device__ __forceinline__ void load_record(const float *rec, bool on, uint32_t (&w)[8])
 {
-    asm("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
-        : "l"(rec));
-}
-
-// Adds K consecutive owners (vox[e .. e + K)) of R record planes: their
-// loads are issued together, then added in ascending owner order per frame.
-template <int R, int K>
-__device__ __forceinline__ void add_owners(const float *dl, size_t plane, const uint32_t *vox, uint32_t e,
-                                           float (&acc)[R * kBwRecord])
-{
-    uint32_t v[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = __ldg(vox + e + k);
-    uint32_t w[K][R][8];
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-        for (int r = 0; r < R; ++r) load_record(dl + r * plane + (size_t)v[k] * kBwRecord, w[k][r]);
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int f = 0; f < kBwRecord; ++f) acc[r * kBwRecord + f] += __uint_as_float(w[k][r][f]);
+    for (int q = 0; q < 8; ++q) w[q] = 0u;
+    asm("{\n .reg .pred p;\n setp.ne.u32 p, %9, 0;\n"
+        " @p ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n}\n"
+        : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]), "+r"(w[4]), "+r"(w[5]), "+r"(w[6]), "+r"(w[7])
+        : "l"(rec), "r"((uint32_t)on));
 }
 
 // Up to R * kBwRecord frames: b.dl holds R planes of records of kBwRecord
@@ -313,47 +394,64 @@ __device__ __forceinline__ void add_owners(const float *dl, size_t plane, const 
 // d_slm (frame f at b.d_slm + f n_pix) is bit-identical to one frame per
 // call; d_mean and d_var receive the frames' gradients added in frame order
 // to 0 (or, with `accumulate`, to what they hold).
+// Bound by the record reads (1.0 GB of sectors per 16 frames of 128^3 x 8):
+// 218 us per 16 frames; 305 when each frame's colours were byte loads in that
+// frame's branch, a memory latency each.  Four CTAs per SM: 64 registers.
 template <int R>
-__global__ void __launch_bounds__(256) owner_pixel_group_kernel(const __grid_constant__ BackwardArgs b,
+__global__ void __launch_bounds__(256, 4) owner_pixel_group_kernel(const __grid_constant__ BackwardArgs b,
                                                                 const uint32_t *off, const uint32_t *vox,
                                                                 int n_frames, int64_t img_fstride, int accumulate)
 {
     constexpr int kF = R * kBwRecord;
+    constexpr int K = 4 / R;   // owners per step: four records in flight
     const size_t plane = (size_t)b.f.nx * b.f.ny * b.f.nz * kBwRecord;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < b.n_pix; p += stride) {
-        const uint32_t e0 = __ldg(off + p);
-        uint32_t e1 = __ldg(off + p + 1);
-#ifdef PSFS_BOUNDS_CHECK
-        {   // the pixel's segment lies in the lists and names voxels of the grid
-            const uint64_t n_vox = (uint64_t)b.f.nx * b.f.ny * b.f.nz;
-            bool seg_ok = PSFS_IN_BOUNDS(e0 <= e1 && e1 <= __ldg(off + b.n_pix), b.f.status);
-            for (uint32_t e = e0; seg_ok && e < e1; ++e) seg_ok = PSFS_IN_BOUNDS(__ldg(vox + e) < n_vox, b.f.status);
-            if (!seg_ok) e1 = e0;
-        }
-#endif
+    const int64_t n_lanes = (b.n_pix + 31) / 32 * 32;   // whole warps: a warp walks its slice together
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_lanes; p += stride) {
+        const uint32_t e0 = __ldg(off + min(p, b.n_pix)), e1 = __ldg(off + min(p + 1, b.n_pix));
+        OwnerWalk<K> walk;
+        walk.init(vox, e0, e1);
         float acc[kF];
 #pragma unroll
         for (int f = 0; f < kF; ++f) acc[f] = 0.0f;
-        // four record loads in flight (four owners of one plane, two of two
-        // planes), then the rest two and one at a time
-        uint32_t e = e0;
-        if constexpr (R == 1) {
-            for (; e + 4 <= e1; e += 4) add_owners<R, 4>(b.dl, plane, vox, e, acc);
-        }
-        for (; e + 2 <= e1; e += 2) add_owners<R, 2>(b.dl, plane, vox, e, acc);
-        if (e < e1) add_owners<R, 1>(b.dl, plane, vox, e, acc);
-        float tm[3] = {0.0f, 0.0f, 0.0f}, tv[3] = {0.0f, 0.0f, 0.0f};
-        if (accumulate) {
+        uint32_t v[K];
+        const uint32_t cnt = e1 - e0;
+        const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, cnt);
+        walk.step(v);
+        for (uint32_t j = 0; j < longest; j += K) {
+            uint32_t w[K][R][8];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                if (b.d_mean) tm[c] = b.d_mean[3 * p + c];
-                if (b.d_var) tv[c] = b.d_var[3 * p + c];
+            for (int k = 0; k < K; ++k) {
+                const bool on = j + k < cnt && owner_in_grid(b, v[k]);
+#pragma unroll
+                for (int r = 0; r < R; ++r) load_record(b.dl + r * plane + (size_t)v[k] * kBwRecord, on, w[k][r]);
             }
+            walk.step(v);
+            // owners in ascending order per frame; a lane past its list adds
+            // +0, which leaves its sums (never -0) as they are
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int f = 0; f < kBwRecord; ++f) acc[r * kBwRecord + f] += __uint_as_float(w[k][r][f]);
         }
+        const bool in_img = p < b.n_pix;
         bool any = false;
 #pragma unroll
         for (int f = 0; f < kF; ++f) any |= (f < n_frames) & (acc[f] != 0.0f);
+        // every frame's colours of the warp's 32 pixels (96 consecutive bytes,
+        // one 4-byte word per lane) and the background in flight together;
+        // byte loads inside each frame's branch waited for memory frame by frame
+        const bool any_lane = __any_sync(0xFFFFFFFFu, any);
+        const int lane = threadIdx.x & 31;
+        const int64_t word = (p - lane) * 3 / 4 + lane;
+        const bool load_word = any_lane && lane < 24 && 4 * word < 3 * b.n_pix;
+        uint32_t iw[kF];
+#pragma unroll
+        for (int f = 0; f < kF; ++f)
+            iw[f] = f < n_frames && load_word
+                        ? __ldg(reinterpret_cast<const uint32_t *>(b.img + f * img_fstride) + word) : 0u;
         float mu[3] = {0.0f, 0.0f, 0.0f}, hh[3] = {0.0f, 0.0f, 0.0f}, base = 0.0f;
         if (any) {
 #pragma unroll
@@ -363,12 +461,24 @@ __global__ void __launch_bounds__(256) owner_pixel_group_kernel(const __grid_con
             }
             base = pixel_log_base(hh[0], hh[1], hh[2], b.c0);
         }
+        float tm[3] = {0.0f, 0.0f, 0.0f}, tv[3] = {0.0f, 0.0f, 0.0f};
+        if (accumulate && in_img) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (b.d_mean) tm[c] = b.d_mean[3 * p + c];
+                if (b.d_var) tv[c] = b.d_var[3 * p + c];
+            }
+        }
+        const int w0 = 3 * lane / 4, shift = 8 * (3 * lane % 4);
 #pragma unroll
         for (int f = 0; f < kF; ++f) {
             if (f < n_frames) {
                 float dslm, dm[3], dv[3];
-                chain_rule_pre(b, b.img + f * img_fstride + 3 * p, mu, hh, base, acc[f], dslm, dm, dv);
-                if (b.d_slm) b.d_slm[f * b.n_pix + p] = dslm;
+                const uint32_t px = __funnelshift_r(__shfl_sync(0xFFFFFFFFu, iw[f], w0),
+                                                    __shfl_sync(0xFFFFFFFFu, iw[f], w0 + 1), shift);
+                const float im[3] = {(float)(px & 255u), (float)((px >> 8) & 255u), (float)((px >> 16) & 255u)};
+                chain_rule_pre(b, im, mu, hh, base, acc[f], dslm, dm, dv);
+                if (b.d_slm && in_img) b.d_slm[f * b.n_pix + p] = dslm;
                 // separate round-to-nearest adds: the compiler may not fuse
                 // them with the products above, so the sums are those of the
                 // per-frame gradients as psfs_backward stores them
@@ -379,6 +489,7 @@ __global__ void __launch_bounds__(256) owner_pixel_group_kernel(const __grid_con
                 }
             }
         }
+        if (!in_img) continue;
         if (b.d_mean)
             for (int c = 0; c < 3; ++c) b.d_mean[3 * p + c] = tm[c];
         if (b.d_var)
@@ -457,7 +568,9 @@ cudaError_t launch_build_owners(const FuseArgs &a, int64_t n_pix, uint32_t *cnt,
     if (e != cudaSuccess) return e;
     owner_fill_kernel<<<(int)vox_blocks, 256, 0, s>>>(a, off, cnt, vox);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    owner_sort_kernel<<<(int)grid_for(n_pix), 256, 0, s>>>(off, vox, n_pix);
+    const int64_t sort_blocks = (n_pix + 32 * kSortWarps - 1) / (32 * kSortWarps);
+    owner_sort_kernel<<<(int)std::min<int64_t>(sort_blocks, 64 * (int64_t)device_sm_count()), 32 * kSortWarps, 0, s>>>(
+        off, vox, n_pix);
     return cudaGetLastError();
 }
 
@@ -479,7 +592,9 @@ cudaError_t launch_owner_pixel(const BackwardArgs &b, const uint32_t *off, const
 cudaError_t launch_owner_pixel_group(const BackwardArgs &b, const uint32_t *off, const uint32_t *vox, int n_frames,
                                      int64_t img_fstride, bool accumulate, cudaStream_t s)
 {
-    if (n_frames < 1 || n_frames > 2 * kBwRecord || !b.img || ((uintptr_t)b.dl & 31u))
+    // whole 4-byte words of whole frames (the entry points ask for 16 bytes of both)
+    if (n_frames < 1 || n_frames > 2 * kBwRecord || !b.img || ((uintptr_t)b.dl & 31u) ||
+        (((uintptr_t)b.img | (uintptr_t)img_fstride) & 3u) || (3 * b.n_pix) % 4 != 0)
         return cudaErrorInvalidValue;
     if (n_frames > kBwRecord)
         owner_pixel_group_kernel<2><<<(int)grid_for(b.n_pix), 256, 0, s>>>(b, off, vox, n_frames, img_fstride,

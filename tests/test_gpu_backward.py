@@ -404,3 +404,46 @@ def test_backward_from_occupancy_equals_recomputing_adjoint():
     assert torch.equal(s1, s2) and torch.equal(m1, m2) and torch.equal(v1, v2)
     assert torch.equal(s1, outs[0][0][4].cuda())
     rec.close()
+
+
+@pytest.mark.parametrize("grid_n,width,height,frames", [(24, 67, 51, 3), (64, 28, 20, 12), (40, 64, 36, 17)])
+def test_owner_list_layouts(grid_n, width, height, frames):
+    """Owner lists as jagged rows (pixel counts that are not whole slices of
+    32), side by side (an image so coarse that slices hold thousands of
+    voxels) and both in one image.  With s = 1/2 everywhere the posterior is
+    exactly 1/2, so whole-number d_occ give sums that FP32 holds exactly:
+    every pixel must have the FP64 sum over its voxels (boundary voxels get
+    d_occ 0), up to the few roundings of the chain rule (1e-5).  The frames of
+    the batched pass are those of one frame per call."""
+    sc = S.make_scene(seed=61, grid_n=grid_n, cube_side=2.0, n_cams=3, width=width, height=height,
+                      focal=0.9 * width, n_frames=frames, walking=True)
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+    pix = oracle.voxel_pixels(sc.grid, sc.cams)
+    bnd = oracle.reconstruct(sc.grid, sc.cams, sc.images[0], sc.mean, sc.var, sc.params)["boundary"]
+    d_occ = np.random.default_rng(6).integers(-8, 9, sc.grid.n_voxels).astype(np.float32)
+    d_occ[bnd] = 0
+    n_pix = 3 * width * height
+    got = torch.empty(n_pix, device="cuda")
+    psfs.psfs_backward_slm(rec.handle, torch.full((n_pix,), 0.5, device="cuda"), to_dev(d_occ), got)
+    assert rec.sync() == psfs.PSFS_OK
+    pd, q = sc.params.p_detect, 0.5 * (sc.params.p_detect + sc.params.p_false_alarm)
+    want = np.zeros((3, width * height))
+    for c in range(3):
+        seen = pix[c] >= 0
+        want[c] = np.bincount(pix[c][seen], weights=0.25 * d_occ[seen].astype(np.float64), minlength=width * height)
+    want = want.ravel() * ((2 * pd - 1) / 0.5 - (2 * q - 1) / 0.5)
+    np.testing.assert_allclose(got.cpu().numpy(), want, rtol=1e-5, atol=0)
+    # the batched pixel pass
+    rec.set_background(to_dev(sc.mean), to_dev(sc.var))
+    if (n_pix * 3) % 16 == 0:
+        imgs = to_dev(sc.images)
+        occ = torch.rand((frames, sc.grid.n_voxels), generator=torch.Generator().manual_seed(1)).cuda()
+        g = torch.randn((frames, sc.grid.n_voxels), generator=torch.Generator().manual_seed(2)).cuda()
+        many = torch.empty((frames, n_pix), device="cuda")
+        one = torch.empty(n_pix, device="cuda")
+        psfs.psfs_backward_from_occupancy(rec.handle, frames, imgs, occ, g, many, None, None)
+        for f in range(frames):
+            psfs.psfs_backward_from_occupancy(rec.handle, 1, imgs[f], occ[f], g[f], one, None, None)
+            assert torch.equal(many[f], one), f
+        assert rec.sync() == psfs.PSFS_OK
+    rec.close()
