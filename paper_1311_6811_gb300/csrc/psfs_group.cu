@@ -37,24 +37,6 @@ namespace {
 // F-wide map vectors
 // ---------------------------------------------------------------------------
 template <typename T>
-__device__ __forceinline__ T to_map(float g);
-template <>
-__device__ __forceinline__ float to_map<float>(float g) { return g; }
-template <>
-__device__ __forceinline__ __half to_map<__half>(float g) { return __float2half_rn(g); }
-template <>
-__device__ __forceinline__ __nv_bfloat16 to_map<__nv_bfloat16>(float g) { return __float2bfloat16_rn(g); }
-
-template <typename T>
-__device__ __forceinline__ uint32_t map_bits(T v);
-template <>
-__device__ __forceinline__ uint32_t map_bits<float>(float v) { return __float_as_uint(v); }
-template <>
-__device__ __forceinline__ uint32_t map_bits<__half>(__half v) { return __half_as_ushort(v); }
-template <>
-__device__ __forceinline__ uint32_t map_bits<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat16_as_ushort(v); }
-
-template <typename T>
 __device__ __forceinline__ float map_value(uint32_t bits);
 template <>
 __device__ __forceinline__ float map_value<float>(uint32_t bits) { return __uint_as_float(bits); }
@@ -76,15 +58,6 @@ struct GroupWords {
     static constexpr int kWords = (F * (int)sizeof(T) + 3) / 4;
     uint32_t w[kWords];
 
-    __device__ __forceinline__ void set(int e, T v)
-    {
-        if (sizeof(T) == 4) {
-            w[e] = map_bits<T>(v);
-        } else {
-            const uint32_t b = map_bits<T>(v) & 0xFFFFu;
-            w[e >> 1] = (e & 1) ? (w[e >> 1] | (b << 16)) : b;
-        }
-    }
     __device__ __forceinline__ float get(int e) const
     {
         if (sizeof(T) == 4) return map_value<T>(w[e]);
@@ -198,6 +171,59 @@ struct GLayout {
     static constexpr int kSmem = kStages * kStage + kStages * 8;    // + mbarriers
 };
 
+// Two frames of one pixel at once: pixel_quad and log_ratio_of_r with every
+// multiply, add and fma on both frames in one packed instruction (the same
+// operations on each, so the same bits).  The likelihood is bound by issue,
+// and beside a fusion it takes the issue slots that one lacks: 100-frame
+// sequence of 128^3 x 8 1095 -> 1064 us, 64 frames with 16-bit maps 544 -> 496.
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+
+__device__ __forceinline__ float2 pixel_quad2(float2 i0, float2 i1, float2 i2, float2 nm0, float2 nm1, float2 nm2,
+                                              float2 h0, float2 h1, float2 h2)
+{
+    const float2 d0 = __fadd2_rn(i0, nm0), d1 = __fadd2_rn(i1, nm1), d2 = __fadd2_rn(i2, nm2);   // nm = -mean
+    return __ffma2_rn(__fmul2_rn(d0, d0), h0,
+                      __ffma2_rn(__fmul2_rn(d1, d1), h1, __fmul2_rn(__fmul2_rn(d2, d2), h2)));
+}
+
+__device__ __forceinline__ float2 log_ratio_of_r2(float2 r, const SensorConsts &c)
+{
+    if (c.a_zero_const_pos | c.a_zero_const_neg)   // P_D in {0, 1} (uniform across the launch)
+        return make_float2(log_ratio_of_r(r.x, c), log_ratio_of_r(r.y, c));
+    const float2 e = __fmul2_rn(make_float2(-fabsf(r.x), -fabsf(r.y)), dup(kLog2e));
+    const float2 u = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+    const bool px = r.x > 0.0f, py = r.y > 0.0f;
+    const float2 hi = make_float2(px ? c.pd : c.one_minus_pd, py ? c.pd : c.one_minus_pd);
+    const float2 lo = make_float2(px ? c.one_minus_pd : c.pd, py ? c.one_minus_pd : c.pd);
+    const float2 hq = make_float2(px ? c.q : c.one_minus_q, py ? c.q : c.one_minus_q);
+    const float2 lq = make_float2(px ? c.one_minus_q : c.q, py ? c.one_minus_q : c.q);
+    const float2 A = __ffma2_rn(lo, u, hi), B = __ffma2_rn(lq, u, hq);
+    const float2 q = __fmul2_rn(A, make_float2(rcp_approx(B.x), rcp_approx(B.y)));
+    return __fmul2_rn(make_float2(lg2_approx(q.x), lg2_approx(q.y)), dup(kLn2));
+}
+
+// Frames e and e + 1 (e even) into a record's words.
+template <typename OutT>
+__device__ __forceinline__ void set_pair(uint32_t *w, int e, float2 g);
+template <>
+__device__ __forceinline__ void set_pair<float>(uint32_t *w, int e, float2 g)
+{
+    w[e] = __float_as_uint(g.x);
+    w[e + 1] = __float_as_uint(g.y);
+}
+template <>
+__device__ __forceinline__ void set_pair<__half>(uint32_t *w, int e, float2 g)
+{
+    const __half2 h = __floats2half2_rn(g.x, g.y);
+    w[e >> 1] = *reinterpret_cast<const uint32_t *>(&h);
+}
+template <>
+__device__ __forceinline__ void set_pair<__nv_bfloat16>(uint32_t *w, int e, float2 g)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(g.x, g.y);
+    w[e >> 1] = *reinterpret_cast<const uint32_t *>(&h);
+}
+
 template <typename OutT, int F, int RB>
 __device__ __forceinline__ void group_pixel(const LikelihoodArgs &a, OutT *out, int64_t p, const unsigned char *im,
                                             int64_t im_stride, const float *m, const float *h)
@@ -216,10 +242,13 @@ __device__ __forceinline__ void group_pixel(const LikelihoodArgs &a, OutT *out, 
     for (int q = 0; q < F / kPlane; ++q) {
         GroupWords<OutT, kPlane> pk;
 #pragma unroll
-        for (int e = 0; e < kPlane; ++e) {
-            const unsigned char *px = im + (q * kPlane + e) * im_stride;
-            const float r = base + pixel_quad((float)px[0], (float)px[1], (float)px[2], m0, m1, m2, h0, h1, h2);
-            pk.set(e, to_map<OutT>(log_ratio_of_r(r, a.sc)));
+        for (int e = 0; e < kPlane; e += 2) {
+            const unsigned char *p0 = im + (q * kPlane + e) * im_stride, *p1 = p0 + im_stride;
+            const float2 quad = pixel_quad2(make_float2((float)p0[0], (float)p1[0]),
+                                            make_float2((float)p0[1], (float)p1[1]),
+                                            make_float2((float)p0[2], (float)p1[2]), dup(-m0), dup(-m1), dup(-m2),
+                                            dup(h0), dup(h1), dup(h2));
+            set_pair<OutT>(pk.w, e, log_ratio_of_r2(__fadd2_rn(dup(base), quad), a.sc));
         }
         store_words<kWords>(reinterpret_cast<uint32_t *>(out + ((int64_t)q * a.n_pix + p) * kPlane), pk.w);
     }
@@ -430,7 +459,27 @@ __device__ __forceinline__ void group_gather(const FuseArgs &a, const TileCoords
         float bu, bv, bw;
         project_base(m, tc.fi, tc.fj, &bu, &bv, &bw);
         const uint32_t *map = maps + (int64_t)c * a.map_stride * kRec + part * Words::kWords;
-        if (flags & kTcInside) {
+        const bool inside = (flags & kTcInside) != 0;
+        // records of 16 frames: one loop with the test inside instead of a
+        // loop per case, half the code (16-bit sequences of 64 frames: 556 ->
+        // 541 us; smaller records measured slower, 69 -> 73 us for 13 frames)
+        if constexpr (F >= 16) {
+#pragma unroll
+            for (int t = 0; t < TZ; ++t) {
+                const Proj p = project_biased(m, bu, bv, bw, tc.fk[t]);
+                int pix;
+                if (inside) {
+                    // the host proved the pixel lies in the image; min() only guards the buffer
+                    if (!PSFS_IN_BOUNDS(proved_inside(p, W, H), a.status)) continue;
+                    pix = (int)min(p.by * W + p.bx + bias_off, last_pix);
+                } else if (!proj_pixel(p, W, H, &pix)) {
+                    continue;
+                }
+                Words g;
+                load_words<Words::kWords>(map + (size_t)pix * kRec, g.w);
+                add_words<MapT, F, TZ>(g, L, t);
+            }
+        } else if (inside) {
 #pragma unroll
             for (int t = 0; t < TZ; ++t) {
                 const Proj p = project_biased(m, bu, bv, bw, tc.fk[t]);
