@@ -62,9 +62,12 @@ __global__ void __launch_bounds__(kSurfThreads) surface_test_kernel(SurfaceArgs 
             v = __ldg(list + e);
             if (v < a.n_vox) {
                 const uint32_t k = v / nxy, r = v - k * nxy, j = r / nx, i = r - j * nx;
-                surf = i == 0 || i + 1 == nx || j == 0 || j + 1 == ny || k == 0 || k + 1 == nz ||
-                       !mask_bit(mask, v - 1) || !mask_bit(mask, v + 1) || !mask_bit(mask, v - nx) ||
-                       !mask_bit(mask, v + nx) || !mask_bit(mask, v - nxy) || !mask_bit(mask, v + nxy);
+                surf = i == 0 || i + 1 == nx || j == 0 || j + 1 == ny || k == 0 || k + 1 == nz;
+                // all six probes in flight together (one after the other, a
+                // voxel inside the body waited for memory six times)
+                if (!surf)
+                    surf = !(mask_bit(mask, v - 1) & mask_bit(mask, v + 1) & mask_bit(mask, v - nx) &
+                             mask_bit(mask, v + nx) & mask_bit(mask, v - nxy) & mask_bit(mask, v + nxy));
             }
         }
         const uint32_t b = __ballot_sync(0xFFFFFFFFu, surf);
@@ -86,12 +89,11 @@ cudaError_t launch_surface(const SurfaceArgs &a, int n_frames, cudaStream_t s)
     if (n_frames <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(a.masks, 0, (size_t)n_frames * a.mask_words * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    // blocks per frame: about four per SM in total (a handful of frames
-    // still fills the GPU), at most one per 256 list entries
-    int sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const uint32_t want = (uint32_t)std::max(1, 4 * std::max(sms, 1) / n_frames);
+    // blocks per frame: about eight per SM in total, all that fit (both passes
+    // wait for memory; a handful of frames still fills the GPU), at most one
+    // per 256 list entries.  100 frames of 15 K voxels: 41.5 ->
+    // 39.4 us with this and the probes together.
+    const uint32_t want = (uint32_t)std::max(1, 8 * std::max(device_sm_count(), 1) / n_frames);
     const uint32_t per_frame =
         std::max<uint32_t>(1, std::min<uint32_t>(std::min<uint32_t>(want, 64), (a.list_stride + kSurfThreads - 1) / kSurfThreads));
     const dim3 grid(per_frame, (unsigned)n_frames);
