@@ -23,16 +23,18 @@ namespace psfs {
 namespace {
 
 template <typename MapT, int LX, int WY, int TZ>
-__global__ void __launch_bounds__(32 * WY) backward_voxel_kernel(const __grid_constant__ BackwardArgs b)
+__global__ void __launch_bounds__(32 * WY) backward_voxel_kernel(const __grid_constant__ BackwardArgs b,
+                                                                 int parts_log2)
 {
     const FuseArgs &a = b.f;
     __shared__ int s_flags[PSFS_MAX_CAMS];
     const int lane = threadIdx.x;
     const int wy = threadIdx.y;
     const int tid = wy * 32 + lane;
-    if (tid < a.n_cams) s_flags[tid] = __ldg(&a.tilecam[(int64_t)blockIdx.x * a.n_cams + tid].w) >> 16;
+    const uint32_t tile = blockIdx.x >> parts_log2;
+    if (tid < a.n_cams) s_flags[tid] = __ldg(&a.tilecam[(int64_t)tile * a.n_cams + tid].w) >> 16;
     TileCoords<LX, WY, TZ> tc;
-    tc.init(a, a.tiles[blockIdx.x], lane, wy);
+    tc.init(a, a.tiles[tile], lane, wy, 1 << parts_log2, (int)(blockIdx.x - (tile << parts_log2)));
     const uint32_t W = (uint32_t)a.W, H = (uint32_t)a.H;
     float L[TZ];
 #pragma unroll
@@ -62,37 +64,32 @@ __global__ void __launch_bounds__(32 * WY) backward_voxel_kernel(const __grid_co
 }
 
 template <typename MapT, int LX, int TZ>
-cudaError_t launch_voxel_typed(const BackwardArgs &b, cudaStream_t s)
+cudaError_t launch_voxel_typed(const BackwardArgs &b, int parts_log2, cudaStream_t s)
 {
-    backward_voxel_kernel<MapT, LX, 4, TZ><<<b.f.n_tiles, dim3(32, 4), 0, s>>>(b);
+    backward_voxel_kernel<MapT, LX, 4, TZ><<<(unsigned)b.f.n_tiles << parts_log2, dim3(32, 4), 0, s>>>(b, parts_log2);
     return cudaGetLastError();
+}
+
+template <typename MapT, int LX>
+cudaError_t launch_voxel_lx(const BackwardArgs &b, int tz, cudaStream_t s)
+{
+    const int p = tile_parts_log2(b.f.n_tiles, tz);
+    switch (tz >> p) {
+    case 2: return launch_voxel_typed<MapT, LX, 2>(b, p, s);
+    case 4: return launch_voxel_typed<MapT, LX, 4>(b, p, s);
+    case 8: return launch_voxel_typed<MapT, LX, 8>(b, p, s);
+    case 16: return launch_voxel_typed<MapT, LX, 16>(b, p, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <typename MapT>
 cudaError_t launch_voxel_shape(const BackwardArgs &b, const FuseShape &sh, cudaStream_t s)
 {
     if (sh.wy != 4) return cudaErrorInvalidValue;
-    if (sh.lx == 8) {
-        if (sh.tz == 2) return launch_voxel_typed<MapT, 8, 2>(b, s);
-        if (sh.tz == 4) return launch_voxel_typed<MapT, 8, 4>(b, s);
-        if (sh.tz == 8) return launch_voxel_typed<MapT, 8, 8>(b, s);
-        if (sh.tz == 16) return launch_voxel_typed<MapT, 8, 16>(b, s);
-        return cudaErrorInvalidValue;
-    }
-    if (sh.lx == 16) {
-        if (sh.tz == 2) return launch_voxel_typed<MapT, 16, 2>(b, s);
-        if (sh.tz == 4) return launch_voxel_typed<MapT, 16, 4>(b, s);
-        if (sh.tz == 8) return launch_voxel_typed<MapT, 16, 8>(b, s);
-        if (sh.tz == 16) return launch_voxel_typed<MapT, 16, 16>(b, s);
-        return cudaErrorInvalidValue;
-    }
-    if (sh.lx == 32) {
-        if (sh.tz == 2) return launch_voxel_typed<MapT, 32, 2>(b, s);
-        if (sh.tz == 4) return launch_voxel_typed<MapT, 32, 4>(b, s);
-        if (sh.tz == 8) return launch_voxel_typed<MapT, 32, 8>(b, s);
-        if (sh.tz == 16) return launch_voxel_typed<MapT, 32, 16>(b, s);
-        return cudaErrorInvalidValue;
-    }
+    if (sh.lx == 8) return launch_voxel_lx<MapT, 8>(b, sh.tz, s);
+    if (sh.lx == 16) return launch_voxel_lx<MapT, 16>(b, sh.tz, s);
+    if (sh.lx == 32) return launch_voxel_lx<MapT, 32>(b, sh.tz, s);
     return cudaErrorInvalidValue;
 }
 

@@ -29,8 +29,13 @@ namespace psfs {
 
 namespace {
 
+// FP32 maps with 16 planes per thread are held to 64 registers (8 CTAs per SM
+// instead of 6): beside other frames' kernels the occupancy is worth more than
+// the 8 bytes of spills (batches of 16 rigs 650 -> 641 us; alone 18.5 -> 18.9 us
+// a frame).  16-bit maps the other way round: 256^3 x 16 takes 114 us with
+// the compiler's own 72 registers, 124 with 64 (and 133 with more than 72).
 template <typename MapT, int LX, int WY, int TZ>
-__global__ void __launch_bounds__(32 * WY) fuse_kernel(const __grid_constant__ FuseArgs a)
+__global__ void __launch_bounds__(32 * WY, sizeof(MapT) == 4 && TZ == 16 ? 8 : 0) fuse_kernel(const __grid_constant__ FuseArgs a, int parts_log2)
 {
     __shared__ int s_flags[PSFS_MAX_CAMS];
     __shared__ uint32_t s_warp_off[WY];
@@ -39,10 +44,11 @@ __global__ void __launch_bounds__(32 * WY) fuse_kernel(const __grid_constant__ F
     const int lane = threadIdx.x;
     const int wy = threadIdx.y;
     const int tid = wy * 32 + lane;
-    if (tid < a.n_cams) s_flags[tid] = __ldg(&a.tilecam[(int64_t)blockIdx.x * a.n_cams + tid].w) >> 16;
+    const uint32_t tile = blockIdx.x >> parts_log2;
+    if (tid < a.n_cams) s_flags[tid] = __ldg(&a.tilecam[(int64_t)tile * a.n_cams + tid].w) >> 16;
 
     TileCoords<LX, WY, TZ> tc;
-    tc.init(a, a.tiles[blockIdx.x], lane, wy);
+    tc.init(a, a.tiles[tile], lane, wy, 1 << parts_log2, (int)(blockIdx.x - (tile << parts_log2)));
     const uint32_t W = (uint32_t)a.W, H = (uint32_t)a.H;
     float L[TZ];
 #pragma unroll
@@ -50,8 +56,6 @@ __global__ void __launch_bounds__(32 * WY) fuse_kernel(const __grid_constant__ F
     __syncthreads();
 
     const MapT *maps = reinterpret_cast<const MapT *>(a.maps);
-    const uint32_t last_pix = W * H - 1u;
-    const uint32_t bias_off = 0u - (kFloorBias * W + kFloorBias);
     int c = 0;
     while (c < a.n_cams) {
         const int flags = s_flags[c];
@@ -69,19 +73,19 @@ __global__ void __launch_bounds__(32 * WY) fuse_kernel(const __grid_constant__ F
             project_base(m0, tc.fi, tc.fj, &bu0, &bv0, &bw0);
             project_base(m1, tc.fi, tc.fj, &bu1, &bv1, &bw1);
             const MapT *map0 = maps + (int64_t)c * a.map_stride, *map1 = map0 + a.map_stride;
-            float g0[TZ], g1[TZ];
+            typename MapRaw<MapT>::T g0[TZ], g1[TZ];
 #pragma unroll
-            for (int t = 0; t < TZ; ++t) {
-                const Proj p0 = project_biased(m0, bu0, bv0, bw0, tc.fk[t]);
-                const Proj p1 = project_biased(m1, bu1, bv1, bw1, tc.fk[t]);
-                // the host proved both pixels lie in the image; min() only guards the buffer
-                g0[t] = PSFS_IN_BOUNDS(proved_inside(p0, W, H), a.status)
-                            ? map_load<MapT>(map0 + min(p0.by * W + p0.bx + bias_off, last_pix)) : 0.0f;
-                g1[t] = PSFS_IN_BOUNDS(proved_inside(p1, W, H), a.status)
-                            ? map_load<MapT>(map1 + min(p1.by * W + p1.bx + bias_off, last_pix)) : 0.0f;
+            for (int t = 0; t < TZ; t += 2) {
+                const ProjPair p = project_pair(m0, bu0, bv0, bw0, tc.fk[t], tc.fk[t + 1]);
+                const ProjPair q = project_pair(m1, bu1, bv1, bw1, tc.fk[t], tc.fk[t + 1]);
+                gather_inside<MapT, false>(p.a, p.b, map0, W, H, g0[t], g0[t + 1], a.status);
+                gather_inside<MapT, false>(q.a, q.b, map1, W, H, g1[t], g1[t + 1], a.status);
             }
 #pragma unroll
-            for (int t = 0; t < TZ; ++t) L[t] = (L[t] + g0[t]) + g1[t];
+            for (int t = 0; t < TZ; t += 2) {
+                add_raw<MapT>(g0[t], g0[t + 1], L[t], L[t + 1]);
+                add_raw<MapT>(g1[t], g1[t + 1], L[t], L[t + 1]);
+            }
             c += 2;
             continue;
         }
@@ -104,37 +108,32 @@ __global__ void __launch_bounds__(32 * WY) fuse_kernel(const __grid_constant__ F
 namespace {
 
 template <typename MapT, int LX, int TZ>
-cudaError_t launch_typed(const FuseArgs &a, cudaStream_t s)
+cudaError_t launch_typed(const FuseArgs &a, int parts_log2, cudaStream_t s)
 {
-    fuse_kernel<MapT, LX, 4, TZ><<<a.n_tiles, dim3(32, 4), 0, s>>>(a);
+    fuse_kernel<MapT, LX, 4, TZ><<<(unsigned)a.n_tiles << parts_log2, dim3(32, 4), 0, s>>>(a, parts_log2);
     return cudaGetLastError();
+}
+
+template <typename MapT, int LX>
+cudaError_t launch_lx(const FuseArgs &a, int tz, cudaStream_t s)
+{
+    const int p = tile_parts_log2(a.n_tiles, tz);
+    switch (tz >> p) {
+    case 2: return launch_typed<MapT, LX, 2>(a, p, s);
+    case 4: return launch_typed<MapT, LX, 4>(a, p, s);
+    case 8: return launch_typed<MapT, LX, 8>(a, p, s);
+    case 16: return launch_typed<MapT, LX, 16>(a, p, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <typename MapT>
 cudaError_t launch_shape(const FuseArgs &a, const FuseShape &sh, cudaStream_t s)
 {
     if (sh.wy != 4) return cudaErrorInvalidValue;
-    if (sh.lx == 8) {
-        if (sh.tz == 2) return launch_typed<MapT, 8, 2>(a, s);
-        if (sh.tz == 4) return launch_typed<MapT, 8, 4>(a, s);
-        if (sh.tz == 8) return launch_typed<MapT, 8, 8>(a, s);
-        if (sh.tz == 16) return launch_typed<MapT, 8, 16>(a, s);
-        return cudaErrorInvalidValue;
-    }
-    if (sh.lx == 16) {
-        if (sh.tz == 2) return launch_typed<MapT, 16, 2>(a, s);
-        if (sh.tz == 4) return launch_typed<MapT, 16, 4>(a, s);
-        if (sh.tz == 8) return launch_typed<MapT, 16, 8>(a, s);
-        if (sh.tz == 16) return launch_typed<MapT, 16, 16>(a, s);
-        return cudaErrorInvalidValue;
-    }
-    if (sh.lx == 32) {
-        if (sh.tz == 2) return launch_typed<MapT, 32, 2>(a, s);
-        if (sh.tz == 4) return launch_typed<MapT, 32, 4>(a, s);
-        if (sh.tz == 8) return launch_typed<MapT, 32, 8>(a, s);
-        if (sh.tz == 16) return launch_typed<MapT, 32, 16>(a, s);
-        return cudaErrorInvalidValue;
-    }
+    if (sh.lx == 8) return launch_lx<MapT, 8>(a, sh.tz, s);
+    if (sh.lx == 16) return launch_lx<MapT, 16>(a, sh.tz, s);
+    if (sh.lx == 32) return launch_lx<MapT, 32>(a, sh.tz, s);
     return cudaErrorInvalidValue;
 }
 

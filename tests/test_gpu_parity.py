@@ -320,3 +320,31 @@ def test_256cube_16cam_1280x720_two_bodies(dtype):
     if dtype != "f32":
         assert rep["max_abs_err"] < (5e-3 if dtype == "f16" else 5e-2)
         assert rep["set_diff"] < 0.01 * ref["list"].size
+
+
+@pytest.mark.parametrize("dims", [(40, 33, 29), (9, 70, 50), (64, 64, 64), (130, 120, 35)])
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_tiles_in_parts(dims, dtype):
+    """A grid of few tiles is fused (and its adjoint's voxel pass run) in parts
+    of each tile along z, also where the last tile's later parts lie outside
+    the grid: the bits of tiles of four planes, which are never cut."""
+    base = S.make_scene(seed=71, grid_n=32, cube_side=2.0, n_cams=3, width=160, height=120, focal=150.0)
+    nx, ny, nz = dims
+    vs = 2.0 / max(dims)
+    grid = S.Grid(nx, ny, nz, (-nx * vs / 2, -ny * vs / 2, 0.0), vs)
+    img = to_dev(base.images)
+    d_occ = torch.randn(nx * ny * nz, generator=torch.Generator().manual_seed(3)).cuda()
+    out = []
+    for tz in (4, 8, 16):
+        rec = psfs.Reconstructor(grid, base.cams, base.params, map_dtype=dtype)
+        rec.set_background(to_dev(base.mean), to_dev(base.var))
+        psfs.psfs_set_fuse_config(rec.handle, 8, 4, tz, 0)
+        occ, lst, cnt = rec.reconstruct(img)
+        d_slm = torch.empty(3 * 160 * 120, device="cuda")
+        psfs.psfs_backward(rec.handle, img, d_occ, d_slm, None, None)
+        assert rec.sync() == psfs.PSFS_OK
+        out.append((occ.clone(), np.sort(psfs.voxel_list(lst, cnt, rec.capacity).numpy()), d_slm))
+        rec.close()
+    for o in out[1:]:
+        assert torch.equal(out[0][0], o[0]) and torch.equal(out[0][2], o[2])
+        np.testing.assert_array_equal(out[0][1], o[1])
