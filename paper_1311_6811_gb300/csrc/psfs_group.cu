@@ -380,8 +380,8 @@ __device__ __forceinline__ float2 posterior2(float2 lo)
 // compaction of tile_epilogue (the same per-voxel arithmetic), with the F
 // frames' counts taken together: two barriers per tile, and F threads each
 // reserve one frame's list range with one atomicAdd.  Only warps with an
-// occupied voxel in some frame (few: 1-3 % of the voxels are) form the ballots
-// again to write their lists (100-frame sequence of 128^3 x 8 1064 -> 982 us, 64
+// occupied voxel in some frame (few: 1-3 % of the voxels are) form ballots, for
+// their counts and again for their lists (100-frame sequence of 128^3 x 8 1064 -> 982 us, 64
 // frames with 16-bit maps 496 -> 451).
 template <int WY, int TZ, int F>
 __device__ __forceinline__ void group_epilogue(const FuseArgs &a, int i, int j, int k0, const float (&L)[F][TZ],
@@ -390,29 +390,34 @@ __device__ __forceinline__ void group_epilogue(const FuseArgs &a, int i, int j, 
     const bool in_xy = (i < a.nx) && (j < a.ny);
     const uint32_t zstride = (uint32_t)a.nx * (uint32_t)a.ny;
     const uint32_t lin0 = (uint32_t)i + (uint32_t)a.nx * ((uint32_t)j + (uint32_t)a.ny * (uint32_t)k0);
-    uint32_t warp_total = 0;
+    float top = -INFINITY;   // the largest log-odds of the thread's voxels in any frame
 #pragma unroll
     for (int f = 0; f < F; f += 2) {
         float *occ = a.occ + f * a.occ_fstride;
-        uint32_t c0 = 0, c1 = 0;
 #pragma unroll
         for (int t = 0; t < TZ; ++t) {
-            const bool valid = in_xy && (k0 + t < a.nz);
-            const float2 lo = __fadd2_rn(make_float2(L[f][t], L[f + 1][t]), dup(a.logit_prior));
-            if (valid) {
+            if (in_xy && (k0 + t < a.nz)) {
+                const float2 lo = __fadd2_rn(make_float2(L[f][t], L[f + 1][t]), dup(a.logit_prior));
                 const float2 p = posterior2(lo);
                 float *o = occ + lin0 + (uint32_t)t * zstride;
                 __stcs(o, p.x);
                 __stcs(o + a.occ_fstride, p.y);
+                top = fmaxf(top, fmaxf(lo.x, lo.y));
             }
-            c0 += __popc(__ballot_sync(0xFFFFFFFFu, valid && (lo.x > a.logit_tau)));
-            c1 += __popc(__ballot_sync(0xFFFFFFFFu, valid && (lo.y > a.logit_tau)));
         }
-        if (lane == 0) {
-            s_off[f][wy] = c0;
-            s_off[f + 1][wy] = c1;
+    }
+    const bool hits = __any_sync(0xFFFFFFFFu, top > a.logit_tau);
+    if (hits) {
+#pragma unroll
+        for (int f = 0; f < F; ++f) {
+            uint32_t cnt = 0;
+#pragma unroll
+            for (int t = 0; t < TZ; ++t)
+                cnt += __popc(__ballot_sync(0xFFFFFFFFu, in_xy && (k0 + t < a.nz) && (L[f][t] + a.logit_prior > a.logit_tau)));
+            if (lane == 0) s_off[f][wy] = cnt;
         }
-        warp_total += c0 + c1;
+    } else if (lane < F) {
+        s_off[lane][wy] = 0;
     }
     __syncthreads();
     const int tid = wy * 32 + lane;
@@ -432,7 +437,7 @@ __device__ __forceinline__ void group_epilogue(const FuseArgs &a, int i, int j, 
         s_base[tid] = base;
     }
     __syncthreads();
-    if (!warp_total) return;
+    if (!hits) return;
     const uint32_t lt_mask = (1u << lane) - 1u;
 #pragma unroll
     for (int f = 0; f < F; ++f) {
@@ -560,36 +565,40 @@ __device__ __forceinline__ void pair_epilogue(const FuseArgs &a, int i, int j, i
     const bool in_xy = (i < a.nx) && (j < a.ny);
     const uint32_t zstride = (uint32_t)a.nx * (uint32_t)a.ny;
     const uint32_t lin0 = (uint32_t)i + (uint32_t)a.nx * ((uint32_t)j + (uint32_t)a.ny * (uint32_t)k0);
-    uint32_t warp_total = 0;
+    float top = -INFINITY;
 #pragma unroll
     for (int e = 0; e < FL; e += 2) {
         float *occ = a.occ + (half * FL + e) * a.occ_fstride;
-        uint32_t c_lo[2] = {0, 0}, c_hi[2] = {0, 0};
 #pragma unroll
         for (int t = 0; t < TZ; ++t) {
-            const bool valid = in_xy && (k0 + t < a.nz);
-            const float2 lo = __fadd2_rn(make_float2(L[e][t], L[e + 1][t]), dup(a.logit_prior));
-            if (valid) {
+            if (in_xy && (k0 + t < a.nz)) {
+                const float2 lo = __fadd2_rn(make_float2(L[e][t], L[e + 1][t]), dup(a.logit_prior));
                 const float2 p = posterior2(lo);
                 float *o = occ + lin0 + (uint32_t)t * zstride;
                 __stcs(o, p.x);
                 __stcs(o + a.occ_fstride, p.y);
+                top = fmaxf(top, fmaxf(lo.x, lo.y));
             }
-            const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, valid && (lo.x > a.logit_tau));
-            const uint32_t b1 = __ballot_sync(0xFFFFFFFFu, valid && (lo.y > a.logit_tau));
-            c_lo[0] += __popc(b0 & 0xFFFFu);
-            c_hi[0] += __popc(b0 >> 16);
-            c_lo[1] += __popc(b1 & 0xFFFFu);
-            c_hi[1] += __popc(b1 >> 16);
         }
+    }
+    const bool hits = __any_sync(0xFFFFFFFFu, top > a.logit_tau);
+    if (hits) {
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            if (lane == 0) {
-                s_off[e + d][wy] = c_lo[d];
-                s_off[FL + e + d][wy] = c_hi[d];
+        for (int e = 0; e < FL; ++e) {
+            uint32_t c_lo = 0, c_hi = 0;
+#pragma unroll
+            for (int t = 0; t < TZ; ++t) {
+                const uint32_t b = __ballot_sync(0xFFFFFFFFu, in_xy && (k0 + t < a.nz) && (L[e][t] + a.logit_prior > a.logit_tau));
+                c_lo += __popc(b & 0xFFFFu);
+                c_hi += __popc(b >> 16);
             }
-            warp_total += c_lo[d] + c_hi[d];
+            if (lane == 0) {
+                s_off[e][wy] = c_lo;
+                s_off[FL + e][wy] = c_hi;
+            }
         }
+    } else if (lane < P) {
+        s_off[lane][wy] = 0;
     }
     __syncthreads();
     const int tid = wy * 32 + lane;
@@ -609,7 +618,7 @@ __device__ __forceinline__ void pair_epilogue(const FuseArgs &a, int i, int j, i
         s_base[tid] = base;
     }
     __syncthreads();
-    if (!warp_total) return;
+    if (!hits) return;
     const uint32_t lt_mask = (1u << lane) - 1u;
     const uint32_t half_mask = half ? 0xFFFF0000u : 0x0000FFFFu;
 #pragma unroll
