@@ -826,14 +826,13 @@ def run_ours(args):
         us_rp = 1e3 * t0e.elapsed_time(t1e) / reps / F
         fg = float(masks.float().mean().item())
         rp_bytes = n_pix * 1 + n_surf * 4
-        nxt["reproject"] = {"us_per_frame": us_rp, "frames_per_call": F, "launches_per_call": 2,
+        nxt["reproject"] = {"us_per_frame": us_rp, "frames_per_call": F, "launches_per_call": 1,
                             "surface_voxels_per_frame": n_surf, "silhouette_fraction": fg,
                             "alg_bytes_per_frame": rp_bytes,
                             "achieved_gbs": rp_bytes / (us_rp * 1e-6) / 1e9,
                             "hbm_frac": rp_bytes / (us_rp * 1e-6) / 1e9 / peak_s,
-                            "note": "psfs_reproject of the step's surface lists in one call (mask memset + "
-                                    "1 kernel): one thread per (surface voxel, camera), float32 centre-ray slab "
-                                    "tests over the cube's projected box"}
+                            "note": "psfs_reproject of the step's surface lists in one call (1 kernel): silhouette polygons "
+                                    "of the listed cubes set in a shared-memory bitmask per camera, written once"}
         # tracker weights of 200 particles (10 cylinders each, around frame 0's
         # body) against frame 0's silhouettes
         caps0 = sc.capsules[0]
@@ -858,7 +857,7 @@ def run_ours(args):
         n_samples = n_part * K * len(caps0) * (8 * 4 + 2 * 8)
         nxt["particle_weights"] = {"us_per_call": us_w, "particles": n_part, "cylinders": len(caps0),
                                    "samples_per_call": n_samples, "gsamples_per_s": n_samples / (us_w * 1e-6) / 1e9,
-                                   "note": "psfs_particle_weights (Eq. 14-16), one launch, one CTA per particle; "
+                                   "note": "psfs_particle_weights (Eq. 14-16), one launch, a cluster of CTAs per particle; "
                                            "sample lookups in the L2-resident silhouettes"}
         del masks
         # smoothing + threshold + compaction over the step's occupancy grids
