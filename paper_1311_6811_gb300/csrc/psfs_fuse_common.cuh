@@ -50,9 +50,10 @@ inline int tile_parts_log2(int n_tiles, int tz)
 }
 
 // Posterior 1 / (1 + e^-L) (written to the occupancy grid), strict
-// threshold L > logit(threshold), and compaction: a ballot per z step per
-// warp, one atomicAdd per CTA on the global count, then each warp writes its
-// indices at its prefix offset.  Contains two __syncthreads.
+// threshold L > logit(threshold), and compaction: a ballot per z step in warps
+// that hold an occupied voxel, one atomicAdd per CTA on the global count, then
+// these warps write their indices at their prefix offsets.  Contains two
+// __syncthreads.
 template <int WY, int TZ>
 __device__ __forceinline__ void tile_epilogue_to(const FuseArgs &a, float *occ, uint32_t *list, uint32_t *count,
                                                  int i, int j, int k0, const float *L, int lane, int wy,
