@@ -94,6 +94,8 @@ def lib_path() -> str:
 def load(build_if_missing: bool = True):
     """Load libpsfs.so (building it first if it is missing and nvcc exists)."""
     global _lib
+    if _lib is not None:   # set last, with every signature in place
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -174,14 +176,26 @@ def _check(status: int, func: str):
         raise PsfsError(status, func, msg)
 
 
+_torch = None
+
+
+def _torch_module():
+    """torch, imported on first use (an import statement per argument is a
+    tenth of the host time of a small call)."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
+
+
 def _dev_ptr(x, name: str, dtype=None, numel: Optional[int] = None):
     """Device pointer of a CUDA tensor (checked) or a raw integer / None."""
     if x is None:
         return None
     if isinstance(x, int):
         return x
-    import torch
-    if not isinstance(x, torch.Tensor):
+    if not isinstance(x, _torch_module().Tensor):
         raise TypeError(f"{name}: expected a CUDA tensor or an int pointer")
     if not x.is_cuda:
         raise ValueError(f"{name}: tensor must be on a CUDA device")
@@ -292,7 +306,7 @@ def psfs_set_background(h: int, mean, var):
 
 
 def psfs_reconstruct(h: int, images, occupancy, voxel_list, capacity: int, count):
-    import torch
+    torch = _torch_module()
     _check(load().psfs_reconstruct(h, _dev_ptr(images, "images", torch.uint8),
                                    _dev_ptr(occupancy, "occupancy", torch.float32),
                                    _dev_ptr(voxel_list, "voxel_list"), int(capacity),
