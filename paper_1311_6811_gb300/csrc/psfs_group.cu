@@ -36,35 +36,13 @@ namespace {
 // ---------------------------------------------------------------------------
 // F-wide map vectors
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ float map_value(uint32_t bits);
-template <>
-__device__ __forceinline__ float map_value<float>(uint32_t bits) { return __uint_as_float(bits); }
-template <>
-__device__ __forceinline__ float map_value<__half>(uint32_t bits)
-{
-    return __half2float(__ushort_as_half((unsigned short)bits));
-}
-template <>
-__device__ __forceinline__ float map_value<__nv_bfloat16>(uint32_t bits)
-{
-    return __bfloat162float(__ushort_as_bfloat16((unsigned short)bits));
-}
-
 // Packs F map values into 32-bit words (element e in the low half first for
 // 16-bit types, the little-endian order of a [F] array).
 template <typename T, int F>
 struct GroupWords {
     static constexpr int kWords = (F * (int)sizeof(T) + 3) / 4;
     uint32_t w[kWords];
-
-    __device__ __forceinline__ float get(int e) const
-    {
-        if (sizeof(T) == 4) return map_value<T>(w[e]);
-        return map_value<T>((w[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
-    }
 };
-
 
 // L += g for two 16-bit map values packed in one word (low half first), one
 // mixed-precision add each (sm_100+): the 16-bit value is widened exactly
@@ -91,7 +69,7 @@ __device__ __forceinline__ void add_words(const GroupWords<MapT, F> &g, float (&
 {
     if constexpr (sizeof(MapT) == 4) {
 #pragma unroll
-        for (int f = 0; f < F; ++f) L[f][t] += g.get(f);
+        for (int f = 0; f < F; ++f) L[f][t] += __uint_as_float(g.w[f]);
     } else {
         static_assert(F % 2 == 0, "16-bit records hold pairs of frames");
 #pragma unroll

@@ -377,23 +377,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 }
 
 // Map loads through the coherent path, for maps written earlier in the same
-// kernel by other CTAs (the batched kernel); map_load below uses the
-// read-only path, valid when the maps come from an earlier kernel.
+// kernel by other CTAs (the batched kernel).
 __device__ __forceinline__ float map_load_coherent(const float *p) { return *p; }
 __device__ __forceinline__ float map_load_coherent(const __half *p) { return __half2float(*p); }
 __device__ __forceinline__ float map_load_coherent(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
-
-template <typename T>
-__device__ __forceinline__ float map_load(const T *p);
-template <>
-__device__ __forceinline__ float map_load<float>(const float *p) { return __ldg(p); }
-template <>
-__device__ __forceinline__ float map_load<__half>(const __half *p) { return __half2float(__ldg(p)); }
-template <>
-__device__ __forceinline__ float map_load<__nv_bfloat16>(const __nv_bfloat16 *p)
-{
-    return __bfloat162float(__ldg(p));
-}
 
 // r = log U - log N (Eq. 1) for one pixel, from its colour, mean and
 // h = 1 / (2 var):  r = c0 - 0.5 log(h0 h1 h2) + sum_c (I_c - mu_c)^2 h_c,
@@ -470,7 +457,7 @@ struct PixelInv {
 
 // Silhouettes of listed voxels (psfs_reproject.cu): frame f's list at lists +
 // f * list_stride with counts[f] entries; masks [n_frames][n_cams][H][W]
-// bytes (zeroed by the launcher).
+// bytes (every byte is written).
 struct ReprojectArgs {
     CamMat cam[PSFS_MAX_CAMS];
     PixelInv inv[PSFS_MAX_CAMS];
@@ -619,7 +606,7 @@ cudaError_t launch_surface(const SurfaceArgs &a, int n_frames, cudaStream_t s);
 // its list at lists + f * capacity, its count at counts[f] (zeroed by the
 // launcher).
 struct SmoothArgs {
-    CUtensorMap tmap;   // {nx, ny, nz, n_frames} over prob, boxes of 136 x 10 (smooth_tma_kernel)
+    CUtensorMap tmap;   // {nx, ny, nz, n_frames} over prob, boxes of 136 x 18 (smooth_tma_kernel)
     const float *prob;
     float *smoothed;
     uint32_t *lists;
