@@ -470,6 +470,15 @@ struct ReprojectArgs {
     uint32_t n_vox;
     uint32_t *status;   // status word (bounds-checked build)
 };
+// How a silhouette call is split over CTAs (see reproject_split).
+struct ReprojectSplit {
+    int bands, band_pix;       // ranges of a camera's pixels, and pixels per range (a multiple of 32)
+    int cluster;               // CTAs of a cluster that takes one band of one mask
+    uint32_t most;             // entries of the longest list that the clusters take
+    int parts, part_threads;   // 0, or the parts of a longer list (a CTA each) and a CTA's threads
+};
+constexpr int kRpBandPixels = 98304 * 8;   // pixels of a CTA's bitmask: 96 KB, two CTAs per SM
+ReprojectSplit reproject_split(int64_t n_pix, int64_t frame_cams, uint32_t list_stride, int sms);
 cudaError_t launch_reproject(const ReprojectArgs &a, int n_frames, cudaStream_t s);
 
 // Particle weights of the tracker (psfs_weights.cu): world -> pixel

@@ -9,10 +9,15 @@
 // per pixel: 38 KB for 640 x 480), so every voxel of the frame's list sets its
 // pixels there, and the finished mask is written out once, as whole bytes,
 // zeros included: no memset before and no read-modify-write of the mask.
-// Images of more than kBandPixels take several CTAs, each a range of pixels;
-// when frames x cameras are few, a cluster of CTAs shares one mask, each with
-// every S-th chunk of the list, and each writes one part of the OR of the S
-// bitmasks, read through distributed shared memory.
+// Images of more than kRpBandPixels take several CTAs, each a range of pixels;
+// when frames x cameras are fewer than the SMs, a cluster of CTAs shares one
+// mask, each with every S-th chunk of the list, and each writes one share of
+// the OR of the S bitmasks, read through distributed shared memory.  Where that
+// still leaves SMs idle, a list that is long (only the GPU knows) is taken by a
+// second kernel instead, in as many parts as CTAs are resident: each part's
+// pixels are OR-ed into the mask, which the first kernel's clusters then only
+// fill with zeros, beside the second kernel's projections (see
+// reproject_split).
 //
 // One thread per listed voxel, with the forward kernels' matrices.  When
 // all eight cube corners lie in front of the camera, a centre ray meets the
@@ -32,6 +37,7 @@
 // Run on the surface list, the work is proportional to the body's surface;
 // the silhouette of a solid equals that of its surface voxels.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include "psfs_internal.cuh"
@@ -40,9 +46,8 @@ namespace psfs {
 
 namespace {
 
-constexpr int kRpThreads = 512;
-constexpr int kBandPixels = 98304 * 8;   // pixels of a CTA's bitmask: 96 KB, two CTAs per SM
-constexpr int kMaxCluster = 8;
+constexpr int kRpThreads = 512;   // and 64 registers each: two CTAs per SM
+constexpr int kRpMaxCluster = 8;
 
 // Silhouette loops of a unit cube by camera region: entry (rx + 1) + 3 (ry +
 // 1) + 9 (rz + 1), r = -1 / 0 / +1 for a camera centre below / within /
@@ -108,18 +113,27 @@ SilTable make_sil_table()
     return t;
 }
 
-// Sets the bits lo .. hi (lo <= hi) of a bitmask.  A word that already holds
-// them is only read: bits are never cleared, so a stale read costs an atomic,
-// not a bit.
+// ORs m into a word of a bitmask.  A word that already holds it is only read:
+// bits are never cleared, so a stale read costs an atomic, not a bit.
+__device__ __forceinline__ void or_word(uint32_t *word, uint32_t m)
+{
+    if (m & ~*reinterpret_cast<volatile uint32_t *>(word)) atomicOr(word, m);
+}
+
+// Sets the bits lo .. hi (lo <= hi).  Nearly every run of a voxel's pixels lies
+// in one word, and the others' code is kept out of its way: with one loop over
+// the words 100 frames of 8.4 K voxels, 8 cameras, took 239 us, with this 204.
 __device__ __forceinline__ void set_bits(uint32_t *bits, int lo, int hi)
 {
-    const int w0 = lo >> 5, w1 = hi >> 5;
-    for (int w = w0; w <= w1; ++w) {
-        uint32_t m = 0xFFFFFFFFu;
-        if (w == w0) m <<= lo & 31;
-        if (w == w1) m &= 0xFFFFFFFFu >> (31 - (hi & 31));
-        if (m & ~*reinterpret_cast<volatile uint32_t *>(bits + w)) atomicOr(bits + w, m);
+    uint32_t *w = bits + (lo >> 5), *const last = bits + (hi >> 5);
+    const uint32_t first_m = 0xFFFFFFFFu << (lo & 31), last_m = 0xFFFFFFFFu >> (31 - (hi & 31));
+    if (w == last) {
+        or_word(w, first_m & last_m);
+        return;
     }
+    or_word(w, first_m);
+    for (++w; w < last; ++w) or_word(w, 0xFFFFFFFFu);
+    or_word(last, last_m);
 }
 
 // Division by a run-time constant d: the estimate n floor(2^32 / d) / 2^32 is
@@ -319,50 +333,152 @@ __device__ __forceinline__ uint32_t load_peer(const uint32_t *p, uint32_t rank)
 // The low four bits of v as four bytes of 0 or 1.
 __device__ __forceinline__ uint32_t spread4(uint32_t v) { return ((v & 15u) * 0x00204081u) & 0x01010101u; }
 
-// blockIdx.x = ((camera * bands) + band) * S + rank, blockIdx.y = frame.  The
-// pixels of a camera are numbered row by row; band b holds b * band_pix ..
-// min(W H, (b + 1) band_pix) - 1.
+// Stores the pixels q0 .. q1 - 1 of a band that starts at pixel p0 as bytes
+// (kZero: zeros): single bytes up to the first and after the last whole
+// aligned 16 bytes.
+template <bool kZero>
+__device__ __forceinline__ void store_bits(const uint32_t *bits, uint8_t *mask, int p0, int q0, int q1)
+{
+    if (q0 >= q1) return;
+    const int tid = threadIdx.x;
+    const int head = min(q1 - q0, (int)((16u - (uint32_t)(reinterpret_cast<uintptr_t>(mask + q0) & 15u)) & 15u));
+    const int n16 = (q1 - q0 - head) / 16, tail0 = q0 + head + 16 * n16;
+    for (int u = tid; u < n16; u += (int)blockDim.x) {
+        const int b = q0 + head + 16 * u - p0, w = b >> 5, sh = b & 31;
+        const uint32_t v = kZero ? 0u : __funnelshift_r(bits[w], sh > 16 ? bits[w + 1] : 0u, sh);
+        *reinterpret_cast<uint4 *>(mask + p0 + b) =
+            make_uint4(spread4(v), spread4(v >> 4), spread4(v >> 8), spread4(v >> 12));
+    }
+    if (tid < 32) {
+        const int p = tid < 16 ? q0 + tid : tail0 + tid - 16;
+        if (tid < 16 ? tid < head : p < q1)
+            mask[p] = kZero ? (uint8_t)0 : (uint8_t)((bits[(p - p0) >> 5] >> ((p - p0) & 31)) & 1u);
+    }
+}
+
+// ORs the words wa .. wb of a band's bitmask (`words` words in all, the last
+// one zero) into the band's `n` bytes at dst.  A warp takes 32 words at a time
+// and of these only the groups of four with a set pixel, so that it passes
+// quickly over what its voxels left empty; a lane then has four pixels of a
+// group: one atomic per aligned 4 bytes with a set pixel, next to those of the
+// other lanes, or single bytes where these 4 reach beyond the band.
+__device__ __forceinline__ void or_words(const uint32_t *bits, int wa, int wb, int words, uint8_t *dst, int n)
+{
+    const int lane = threadIdx.x & 31, off = (int)(reinterpret_cast<uintptr_t>(dst) & 3u);
+    // window w: the 32 pixels from pixel 32 w - off on, whose bytes start aligned
+    wb = min(wb + (off ? 1 : 0), words - 1);
+    for (int w0 = wa + (int)(threadIdx.x & ~31u); w0 <= wb; w0 += (int)blockDim.x) {
+        const int w = w0 + lane;
+        const uint32_t hi = w <= wb ? bits[w] : 0u, lo = w <= wb && w > 0 ? bits[w - 1] : 0u;
+        const uint32_t v = __funnelshift_l(lo, hi, off);
+        uint32_t any = __ballot_sync(0xFFFFFFFFu, v != 0u);
+        while (any) {
+            const int g = (__ffs(any) - 1) & ~3;   // words w0 + g .. w0 + g + 3
+            any &= ~(15u << g);
+            const uint32_t q = (__shfl_sync(0xFFFFFFFFu, v, g + (lane >> 3)) >> (4 * (lane & 7))) & 15u;
+            if (!q) continue;
+            const int b = 32 * (w0 + g) + 4 * lane - off;
+            if (b >= 0 && b + 4 <= n) {
+                atomicOr(reinterpret_cast<unsigned int *>(dst + b), spread4(q));
+            } else {
+                for (int k = 0; k < 4; ++k)
+                    if ((q >> k) & 1u) dst[b + k] = 1;
+            }
+        }
+    }
+}
+
+// Programmatic dependent launch: lets the next kernel's CTAs start beside this
+// one's, and in these waits until this one has finished.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void wait_dependency() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
+// blockIdx.y = frame.  The pixels of a camera are numbered row by row; band b
+// holds b * band_pix .. min(W H, (b + 1) band_pix) - 1.
+//   kParts false: blockIdx.x = (camera * bands + band) * n + rank; the n CTAs
+// of a cluster take one mask band and store all its bytes.  Of a frame with
+// more than `most` entries they store zeros; the second kernel takes it.
+//   kParts true: blockIdx.x = (part * n_cams + camera) * bands + band; of a
+// frame with more than `most` entries a CTA takes the part-th of n ranges and
+// ORs its pixels into the zeros of the first kernel, beside which it starts.
+// (Parts outermost: those that a shorter list leaves empty come last.)
 //
-// Bound by issue (about 800 instructions per voxel and camera, most of them
-// the six edge tests of each pixel row): 100 frames of 4.7 K surface voxels, 8
-// cameras of 640 x 480, take 164 us.  Before (chunks of 256 voxels staged as
-// bytes over their common box, OR-ed into a zeroed mask word by word): 275 us;
-// with eight corner depths, corner offsets from selects and integer divisions
-// per voxel instead of the depth bound, the offset table and fast_div: 175 us.
+// 100 frames of 4.7 K surface voxels, 8 cameras of 640 x 480, take 142 us, most
+// of it the six edge tests of each voxel's pixel rows.  Before (chunks of 256
+// voxels staged as bytes over their common box, OR-ed into a zeroed mask word
+// by word): 275 us; with eight corner depths, corner offsets from selects and
+// integer divisions per voxel instead of the depth bound, the offset table and
+// fast_div: 175 us; with a loop over the words of each run in set_bits: 164 us.
+template <bool kParts>
 __global__ void __launch_bounds__(kRpThreads, 2) reproject_kernel(const __grid_constant__ ReprojectArgs a,
                                                                   const __grid_constant__ SilTable sil,
                                                                   FastDiv by_nxy, FastDiv by_nx, int bands,
-                                                                  int band_pix, int S)
+                                                                  int band_pix, int n, uint32_t most)
 {
-    extern __shared__ __align__(16) uint32_t bits[];   // band_pix / 32 words and a zero word
+    extern __shared__ __align__(16) uint32_t bits[];   // band_words(band_pix) words, the last of them zero
+    __shared__ int s_rows[2];                          // kParts: -first, last row with pixels that may be set
     // per camera region the corners of the silhouette loop as offsets from the
     // cube's centre (.w: their number; a 4-corner loop padded with its first)
     __shared__ float4 s_corners[27 * 6];
     const int tid = threadIdx.x;
-    if (tid < 27 * 6) {
-        const uint32_t ent = sil.e[tid / 6], n = ent & 15u, k = tid % 6;
-        const uint32_t q = (ent >> (4 + 3 * (k < n ? k : 0))) & 7u;
-        s_corners[tid] = make_float4((q & 1) ? 0.5f : -0.5f, (q & 2) ? 0.5f : -0.5f, (q & 4) ? 0.5f : -0.5f, (float)n);
-    }
-    const int rank = S == 1 ? 0 : (int)cluster_rank();
-    const int cb = (int)blockIdx.x / S;
+    const int S = kParts ? 1 : n, rank = S == 1 ? 0 : (int)cluster_rank();
+    const int K = a.n_cams, part = kParts ? (int)blockIdx.x / (K * bands) : 0;
+    const int cb = kParts ? (int)blockIdx.x - part * (K * bands) : (int)blockIdx.x / n;
     const int c = cb / bands, f = blockIdx.y;
-    const int K = a.n_cams, W = a.W, n_pix = a.W * a.H;
+    const int W = a.W, n_pix = a.W * a.H;
     const int p0 = (cb - c * bands) * band_pix, p1 = min(n_pix, p0 + band_pix);
+    const int threads = blockDim.x;
+    const uint32_t m_all = min(__ldg(a.counts + f), a.list_stride);
+    const bool is_long = m_all > most;
+    uint8_t *mask = a.masks + ((size_t)f * K + c) * n_pix;
+    // the cluster's share of the band in whole words
+    const int share = ((p1 - p0 + S - 1) / S + 31) & ~31;
+    const int q0 = p0 + rank * share, q1 = min(p1, q0 + share);
+    uint64_t e0 = 0, e1 = m_all;   // this cluster's entries of the list
+    if (kParts) {
+        // equal ranges of whole warps: listed neighbours lie close together, so that a part's pixels overlap
+        const uint32_t per = max((m_all / (uint32_t)n + 32u) & ~31u, 128u);
+        e0 = (uint64_t)part * per;
+        if (!is_long || e0 >= m_all) {
+            if ((blockIdx.x | blockIdx.y) == 0) wait_dependency();   // this grid ends after the first kernel's
+            return;
+        }
+        e1 = min(e0 + per, (uint64_t)m_all);
+        if (tid < 2) s_rows[tid] = INT_MIN;
+    } else {
+        launch_dependents();
+        if (is_long) {
+            store_bits<true>(nullptr, mask, p0, q0, q1);
+            return;
+        }
+    }
+    if (tid < 27 * 6) {
+        const uint32_t ent = sil.e[tid / 6], len = ent & 15u, k = tid % 6;
+        const uint32_t q = (ent >> (4 + 3 * (k < len ? k : 0))) & 7u;
+        s_corners[tid] = make_float4((q & 1) ? 0.5f : -0.5f, (q & 2) ? 0.5f : -0.5f, (q & 4) ? 0.5f : -0.5f, (float)len);
+    }
+    const uint32_t *list = a.lists + (size_t)f * a.list_stride;
+    const uint64_t step = (uint64_t)S * threads;
+    uint64_t e = e0 + (uint64_t)rank * threads + tid;
+    uint32_t next = e < e1 ? __ldg(list + e) : 0u;   // in flight while the bitmask is zeroed
     const int n_words = (p1 - p0 + 31) / 32 + 1;
-    for (int w = tid; w < n_words; w += kRpThreads) bits[w] = 0u;
+    for (int w = tid; w < (n_words + 3) / 4; w += threads) reinterpret_cast<uint4 *>(bits)[w] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
 
-    const uint32_t m_cnt = min(__ldg(a.counts + f), a.list_stride);
-    const uint32_t *list = a.lists + (size_t)f * a.list_stride;
     const int y_lo = p0 / W, y_hi = (p1 - 1) / W;
-    for (uint64_t e = (uint64_t)rank * kRpThreads + tid; e < m_cnt; e += (uint64_t)S * kRpThreads) {
-        const uint32_t v = __ldg(list + e);
+    int ya = INT_MAX, yb = -1;   // rows of this thread's candidate pixels
+    for (; e < e1; e += step) {
+        const uint32_t v = next;
+        if (e + step < e1) next = __ldg(list + e + step);
         if (v >= a.n_vox) continue;
         CubeProj P;
         project_cube(a, s_corners, by_nxy, by_nx, c, v, P);
+        if (P.xa > P.xb) continue;
+        if (kParts) {
+            ya = min(ya, P.ya);
+            yb = max(yb, P.yb);
+        }
         if (P.n >= 3) {
-            if (P.xa > P.xb) continue;
             const int ye = min(P.yb, y_hi);
             for (int y = max(P.ya, y_lo); y <= ye; ++y) {
                 int xs, xe;
@@ -375,88 +491,138 @@ __global__ void __launch_bounds__(kRpThreads, 2) reproject_kernel(const __grid_c
             slab_test_pixels(a, c, P, bits, p0, p1);
         }
     }
+    if (kParts) {
+        ya = __reduce_max_sync(0xFFFFFFFFu, -ya);
+        yb = __reduce_max_sync(0xFFFFFFFFu, yb);
+        if ((tid & 31) == 0) {
+            atomicMax(&s_rows[0], ya);
+            atomicMax(&s_rows[1], yb);
+        }
+        __syncthreads();
+        ya = max(-s_rows[0], y_lo);
+        yb = min(s_rows[1], y_hi);
+        wait_dependency();
+        if (ya <= yb)
+            or_words(bits, max(ya * W - p0, 0) >> 5, (min((yb + 1) * W, p1) - 1 - p0) >> 5, n_words, mask + p0, p1 - p0);
+        return;
+    }
     if (S == 1)
         __syncthreads();
     else
         cluster_sync();
 
-    // this CTA's part of the band: whole words, so that it can OR the peers'
-    // into its own (they read other words of it), then bits as bytes: single
-    // bytes up to the first and after the last whole aligned 16 bytes
-    const int part = ((p1 - p0 + S - 1) / S + 31) & ~31;
-    const int q0 = p0 + rank * part, q1 = min(p1, q0 + part);
+    // this CTA's share of the band: whole words, so that it can OR the peers'
+    // into its own (they read other words of it), then bits as bytes
     if (S > 1) {
-        for (int w = (q0 - p0) / 32 + tid; w < (q1 - p0 + 31) / 32; w += kRpThreads) {
+        for (int w = (q0 - p0) / 32 + tid; w < (q1 - p0 + 31) / 32; w += threads) {
             uint32_t v = 0;
 #pragma unroll
-            for (int r = 0; r < kMaxCluster; ++r)   // independent loads, in flight together
+            for (int r = 0; r < kRpMaxCluster; ++r)   // independent loads, in flight together
                 if (r < S) v |= load_peer(bits + w, (uint32_t)r);
             bits[w] = v;
         }
         __syncthreads();
     }
-    uint8_t *mask = a.masks + ((size_t)f * K + c) * n_pix;
-    if (q0 < q1) {
-        const int head = min(q1 - q0, (int)((16u - (uint32_t)(reinterpret_cast<uintptr_t>(mask + q0) & 15u)) & 15u));
-        const int n16 = (q1 - q0 - head) / 16, tail0 = q0 + head + 16 * n16;
-        for (int u = tid; u < n16; u += kRpThreads) {
-            const int b = q0 + head + 16 * u - p0, w = b >> 5, sh = b & 31;
-            const uint32_t v = __funnelshift_r(bits[w], sh > 16 ? bits[w + 1] : 0u, sh);
-            *reinterpret_cast<uint4 *>(mask + p0 + b) =
-                make_uint4(spread4(v), spread4(v >> 4), spread4(v >> 8), spread4(v >> 12));
-        }
-        if (tid < 32) {
-            const int p = tid < 16 ? q0 + tid : tail0 + tid - 16;
-            if (tid < 16 ? tid < head : p < q1)
-                mask[p] = (uint8_t)((bits[(p - p0) >> 5] >> ((p - p0) & 31)) & 1u);
-        }
-    }
+    store_bits<false>(bits, mask, p0, q0, q1);
     if (S > 1) cluster_sync();   // the peers read this CTA's bitmask until here
 }
 
 }  // namespace
 
-// Bands: as few as hold kBandPixels each (two CTAs per SM).  Cluster size: 1,
-// 2, 4 or 8 CTAs per mask, the smallest that gives four CTAs per SM in all, so
-// that a few frames still fill the GPU (9 frames of 5 cameras, 470 x 351: 18.8
-// us with 8, 24 when each 16 pixels were OR-ed from the peers one load after
-// the other, 27 with the chunked kernel before) and many frames write each mask
-// from one bitmask, without reading peers.
+// Shared memory words of a band's bitmask: its pixels, a zero word, whole 16 bytes.
+static int band_words(int band_pix) { return (band_pix / 32 + 1 + 3) & ~3; }
+
+// Bands: as few as hold kRpBandPixels each (two CTAs per SM).
+//
+// Cluster size: the one with the least time for the SM that gets most CTAs, if
+// a CTA costs 1 / S of a mask's list and 1 / 8 for its bitmask, and CTAs beside
+// each other on an SM 0.82 of that (fitted to 8 to 800 masks and lists of 2.7 K
+// to 43 K voxels; 72 masks of 640 x 480, 8.4 K: 45.9, 29.7, 29.4 and 35.6 us
+// with 1, 2, 4 and 8; 160 masks: 74.7, 65.7, 60.5, 71.0; 800 masks: 204 with 1;
+// sizes that are not powers of two are sometimes placed badly, 24 masks with 6
+// 64 us and with 4 56).
+//
+// Parts, for at most a third as many masks as SMs: four CTAs of 256 threads per
+// SM in all (as shared memory allows).  us with parts / with a cluster per mask
+// only (640 x 480): one mask, 43 K voxels 9.7 / 31.7, 562 K 27 / 290; 8 masks,
+// 43 K 19.6 / 33; 16 masks, 8.4 K 15 / 19.6; 48 masks, 8.4 K 24 / 27.9; 56
+// masks, 8.4 K: the cluster is faster.  Lists of up to 4096 entries, which a
+// cluster of 8 takes in one round, are left to it (8 masks, 4000 voxels in any
+// order 10.8, with parts 10.4 in the grid's order but 14.7 shuffled, as the
+// smoothing leaves them: more atomics), but not where four CTAs per mask do not
+// fit the SMs at once (45 masks, 2.7 K voxels 14.8 / 19.2).
+ReprojectSplit reproject_split(int64_t n_pix, int64_t frame_cams, uint32_t list_stride, int sms)
+{
+    ReprojectSplit r;
+    r.bands = (int)((n_pix + kRpBandPixels - 1) / kRpBandPixels);
+    r.band_pix = (int)(((n_pix + r.bands - 1) / r.bands + 31) & ~(int64_t)31);
+    r.cluster = 1;
+    r.parts = r.part_threads = 0;
+    r.most = UINT32_MAX;
+    const int64_t masks = frame_cams * r.bands;
+    sms = std::max(sms, 1);
+    double best = 1e300;
+    for (int S = 1; S <= kRpMaxCluster; S *= 2) {
+        const int64_t load = (masks * S + sms - 1) / sms;   // CTAs of the fullest SM
+        const double cost = (load == 1 ? 1.0 : 0.82 * (double)load) * (1.0 / S + 0.125);
+        if (cost < best) {
+            best = cost;
+            r.cluster = S;
+        }
+    }
+    const uint32_t most = 4 * masks <= sms ? 4096u : 0u;
+    if (3 * masks <= sms && list_stride > most) {
+        const int per_sm = std::min(4, 220 * 1024 / (4 * band_words(r.band_pix) + 4096));
+        r.most = most;
+        r.parts = (int)std::min<int64_t>(per_sm * (int64_t)sms / masks, ((int64_t)list_stride + 127) / 128);
+        r.part_threads = (2 * kRpThreads / per_sm) & ~31;
+    }
+    return r;
+}
+
 cudaError_t launch_reproject(const ReprojectArgs &a, int n_frames, cudaStream_t s)
 {
     if (n_frames <= 0) return cudaSuccess;
     static const SilTable sil = make_sil_table();
     const int n_pix = a.W * a.H;
-    const int bands = (n_pix + kBandPixels - 1) / kBandPixels;
-    const int band_pix = ((n_pix + bands - 1) / bands + 31) & ~31;
-    const int smem = (band_pix / 32 + 1) * 4;
-    const int64_t masks = (int64_t)n_frames * a.n_cams * bands, want = 4 * (int64_t)std::max(device_sm_count(), 1);
-    int S = 1;
-    while (S < kMaxCluster && masks * S < want) S *= 2;
+    const ReprojectSplit sp = reproject_split(n_pix, (int64_t)n_frames * a.n_cams, a.list_stride, device_sm_count());
     static bool configured[64] = {false};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(reproject_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kBandPixels / 8 + 4);
-        if (e != cudaSuccess) return e;
+        for (const auto k : {reproject_kernel<true>, reproject_kernel<false>}) {
+            const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       4 * band_words(kRpBandPixels));
+            if (e != cudaSuccess) return e;
+        }
         configured[dev] = true;
     }
+    const FastDiv by_nxy = make_fast_div((uint32_t)a.nx * (uint32_t)a.ny), by_nx = make_fast_div((uint32_t)a.nx);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a.n_cams * bands * S), (unsigned)n_frames);
+    cfg.gridDim = dim3((unsigned)(a.n_cams * sp.bands * sp.cluster), (unsigned)n_frames);
     cfg.blockDim = dim3(kRpThreads);
-    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.dynamicSmemBytes = (size_t)(4 * band_words(sp.band_pix));
     cfg.stream = s;
     cudaLaunchAttribute attr = {};
     attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)S;
+    attr.val.clusterDim.x = (unsigned)sp.cluster;
     attr.val.clusterDim.y = 1;
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, reproject_kernel, a, sil, make_fast_div((uint32_t)a.nx * (uint32_t)a.ny),
-                                       make_fast_div((uint32_t)a.nx), bands, band_pix, S);
+    cfg.numAttrs = sp.cluster > 1 ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, reproject_kernel<false>, a, sil, by_nxy, by_nx, sp.bands, sp.band_pix,
+                                       sp.cluster, sp.most);
+    if (e == cudaSuccess && sp.parts) {
+        cfg.gridDim.x = (unsigned)(a.n_cams * sp.bands * sp.parts);
+        cfg.blockDim = dim3((unsigned)sp.part_threads);
+        attr = {};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, reproject_kernel<true>, a, sil, by_nxy, by_nx, sp.bands, sp.band_pix, sp.parts,
+                               sp.most);
+    }
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

@@ -153,3 +153,61 @@ def test_bitmask_bands_and_clusters(width, height, n_cams, frames):
     _check(sc.grid, sc.cams, s_.astype(np.uint32), got[0])
     assert (got == got[0]).all()
     rec.close()
+
+
+@pytest.mark.parametrize("width,height,n_cams,frames,offset", [(67, 51, 2, 1, 0), (67, 51, 2, 3, 1), (33, 1, 1, 3, 3),
+                                                               (64, 48, 3, 2, 2), (1100, 760, 1, 1, 0)])
+def test_parts_of_the_list(width, height, n_cams, frames, offset):
+    """Few masks and lists of more than 4096 entries: parts of the list, a CTA
+    each, OR-ed into a zeroed mask (masks at any byte, rows of any length, two
+    bands; frames with a short and an empty list in the same call).  The masks
+    are the OR of those of the list's pieces, which a cluster per mask takes,
+    against the oracle, and the bytes beside them stay; a captured call gives
+    the same."""
+    sc = S.make_scene(seed=45, grid_n=20, cube_side=2.0, n_cams=n_cams, width=width, height=height,
+                      focal=0.9 * width)
+    stream = torch.cuda.Stream()
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params, stream=stream)
+    rng = np.random.default_rng(6)
+    sizes = [5000, 300, 0][:frames]
+    stride = 5001
+    lists = torch.zeros((frames, stride), dtype=torch.int32)
+    for f, n in enumerate(sizes):
+        lists[f, :n] = torch.from_numpy(np.sort(rng.choice(sc.grid.n_voxels, n, replace=False)).astype(np.int32))
+    n_bytes = frames * n_cams * height * width
+
+    def run(l, s_, c, buf):
+        psfs.psfs_reproject(rec.handle, frames, l, s_, c, buf[offset:offset + n_bytes])
+
+    def masks(buf):
+        assert (buf[:offset] == 7).all() and (buf[offset + n_bytes:] == 7).all()
+        return buf[offset:offset + n_bytes].cpu().numpy().reshape(frames, n_cams, height, width)
+
+    want = np.zeros((frames, n_cams, height, width), np.uint8)
+    for a in range(0, max(sizes), 2500):
+        counts = torch.tensor([min(max(n - a, 0), 2500) for n in sizes], dtype=torch.int32).cuda()
+        buf = torch.full((offset + n_bytes + 5,), 7, dtype=torch.uint8, device="cuda")
+        piece = lists[:, a:a + 2500].contiguous().cuda()
+        torch.cuda.synchronize()
+        run(piece, 2500, counts, buf)
+        assert rec.sync() == psfs.PSFS_OK
+        want |= masks(buf)
+    counts = torch.tensor(sizes, dtype=torch.int32).cuda()
+    dev = lists.cuda()
+    bufs = [torch.full((offset + n_bytes + 5,), 7, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    torch.cuda.synchronize()
+    run(dev, stride, counts, bufs[0])
+    assert rec.sync() == psfs.PSFS_OK
+    got = masks(bufs[0])
+    assert np.array_equal(got, want)
+    if width < 1000:   # the brute force over the large image takes half a minute
+        _check(sc.grid, sc.cams, lists[0, :sizes[0]].numpy().astype(np.uint32), got[0])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        run(dev, stride, counts, bufs[1])
+    with torch.cuda.stream(stream):
+        graph.replay()
+        graph.replay()
+    assert rec.sync() == psfs.PSFS_OK
+    assert np.array_equal(masks(bufs[1]), want)
+    rec.close()
