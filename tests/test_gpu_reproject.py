@@ -211,3 +211,63 @@ def test_parts_of_the_list(width, height, n_cams, frames, offset):
     assert rec.sync() == psfs.PSFS_OK
     assert np.array_equal(masks(bufs[1]), want)
     rec.close()
+
+
+def _depths(grid, cam):
+    """Least and largest depth of every voxel's eight corners in one camera."""
+    z, y, x = np.meshgrid(np.arange(grid.nz), np.arange(grid.ny), np.arange(grid.nx), indexing="ij")
+    i = np.stack([x.ravel(), y.ravel(), z.ravel()], 1).astype(np.float64)
+    corner = np.array([[a, b, c] for a in (0, 1) for b in (0, 1) for c in (0, 1)])
+    X = np.asarray(grid.origin) + (i[:, None, :] + corner[None]) * grid.voxel_size
+    d = X @ cam.R[2] + cam.t[2]
+    return d.min(1), d.max(1)
+
+
+@pytest.mark.parametrize("width,height,frames", [(48, 40, 1), (48, 40, 320), (1100, 760, 1)])
+def test_cubes_at_and_behind_a_camera(width, height, frames):
+    """Cameras inside an 8 m grid: cubes wholly behind one, cubes at its plane
+    (several of one thread, and in rounds of the list beyond its 32nd), in one
+    band and in two, against the oracle."""
+    sc = S.make_scene(seed=46, grid_n=36, cube_side=8.0, n_cams=1, width=width, height=height, focal=0.8 * width)
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+    lo, hi = _depths(sc.grid, sc.cams[0])
+    at, behind, front = (np.flatnonzero(m) for m in ((lo < 0) & (hi > 0), hi < 0, lo > 0))
+    assert at.size > 800 and behind.size > 1000
+    rng = np.random.default_rng(7)
+    n = 800 if width < 1000 else 60
+    s_ = np.concatenate([rng.choice(at, n, replace=False), rng.choice(behind, 100), rng.choice(front, 20)])
+    s_ = rng.permutation(s_).astype(np.int32)
+    if frames > 1:
+        s_ = np.tile(s_, 40)   # more rounds of the list than a thread remembers
+    lists = torch.from_numpy(s_).cuda().repeat(frames, 1)
+    counts = torch.full((frames,), s_.size, dtype=torch.int32, device="cuda")
+    got = _gpu_masks(rec, lists, counts, s_.size)
+    _check(sc.grid, sc.cams, np.unique(s_).astype(np.uint32), got[0])
+    assert (got == got[0]).all()
+    rec.close()
+
+
+def test_cubes_behind_a_camera_cost_no_more_than_those_in_front():
+    """A cube behind a camera meets no ray: it must not be tested against every
+    pixel (that took milliseconds; these lists take about 10 us each, and the
+    bound of ten times leaves room for a disturbed run)."""
+    sc = S.make_scene(seed=47, grid_n=64, cube_side=8.0, n_cams=1, width=320, height=240, focal=250.0)
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+    lo, hi = _depths(sc.grid, sc.cams[0])
+    times = []
+    for m in (lo > 1.0, hi < 0):
+        s_ = np.flatnonzero(m)[:4000].astype(np.int32)
+        lists, counts = torch.from_numpy(s_).cuda().view(1, -1), torch.tensor([s_.size], dtype=torch.int32).cuda()
+        masks = torch.empty((1, 1, 240, 320), dtype=torch.uint8, device="cuda")
+        best = 1e9
+        for _ in range(4):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            psfs.psfs_reproject(rec.handle, 1, lists, s_.size, counts, masks)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        times.append(best)
+    assert rec.sync() == psfs.PSFS_OK
+    assert times[1] <= 10 * times[0], times
+    rec.close()
