@@ -473,11 +473,11 @@ struct ReprojectArgs {
 // How a silhouette call is split over CTAs (see reproject_split).
 struct ReprojectSplit {
     int bands, band_pix;       // ranges of a camera's pixels, and pixels per range (a multiple of 32)
-    int cluster;               // CTAs of a cluster that takes one band of one mask
+    int cluster, threads;      // CTAs of a cluster that takes one band of one mask, and a CTA's threads
     uint32_t most;             // entries of the longest list that the clusters take
     int parts, part_threads;   // 0, or the parts of a longer list (a CTA each) and a CTA's threads
 };
-constexpr int kRpBandPixels = 98304 * 8;   // pixels of a CTA's bitmask: 96 KB, two CTAs per SM
+constexpr int kRpBandPixels = 216 * 1024 * 8;   // most pixels of a CTA's bitmask: 216 KB
 ReprojectSplit reproject_split(int64_t n_pix, int64_t frame_cams, uint32_t list_stride, int sms);
 cudaError_t launch_reproject(const ReprojectArgs &a, int n_frames, cudaStream_t s);
 

@@ -47,7 +47,7 @@ namespace psfs {
 
 namespace {
 
-constexpr int kRpThreads = 512;   // and 64 registers each: two CTAs per SM
+constexpr int kRpSmThreads = 1024;   // of an SM, 64 registers each: one CTA, or two of half, ...
 constexpr int kRpMaxCluster = 8;
 
 // Silhouette loops of a unit cube by camera region: entry (rx + 1) + 3 (ry +
@@ -466,7 +466,7 @@ __device__ __forceinline__ void slab_phase(const ReprojectArgs &a, const float4 
                                         const FastDiv by_nx, int c, const uint32_t *mine, uint64_t step,
                                         uint32_t pending, uint32_t *bits, int p0, int p1)
 {
-    __shared__ uint32_t queue[kRpThreads], queued;
+    __shared__ uint32_t queue[kRpSmThreads], queued;
     do {
         if (threadIdx.x == 0) queued = 0;
         __syncthreads();
@@ -496,7 +496,7 @@ __device__ __forceinline__ void slab_phase(const ReprojectArgs &a, const float4 
 // integer divisions per voxel instead of the depth bound, the offset table and
 // fast_div: 175 us; with a loop over the words of each run in set_bits: 164 us.
 template <bool kParts>
-__global__ void __launch_bounds__(kRpThreads, 2) reproject_kernel(const __grid_constant__ ReprojectArgs a,
+__global__ void __launch_bounds__(kRpSmThreads, 1) reproject_kernel(const __grid_constant__ ReprojectArgs a,
                                                                   const __grid_constant__ SilTable sil,
                                                                   FastDiv by_nxy, FastDiv by_nx, int bands,
                                                                   int band_pix, int n, uint32_t most)
@@ -614,10 +614,20 @@ __global__ void __launch_bounds__(kRpThreads, 2) reproject_kernel(const __grid_c
 
 }  // namespace
 
+constexpr int kRpSmShared = 224 * 1024;   // shared memory of an SM's CTAs
+constexpr int kRpStatic = 8192;           // of a CTA beside its bitmask, no less
+
 // Shared memory words of a band's bitmask: its pixels, a zero word, whole 16 bytes.
 static int band_words(int band_pix) { return (band_pix / 32 + 1 + 3) & ~3; }
 
-// Bands: as few as hold kRpBandPixels each (two CTAs per SM).
+// Bands: as few as hold kRpBandPixels each, because every band projects the
+// whole list again and the body's rows are seldom shared out evenly; CTAs of
+// 512 threads where two of them fit an SM, of 1024 otherwise.  36 masks, 43 K
+// voxels: 1280 x 720 75 us in one band, 114 in two of 96 KB and 512 threads;
+// 1920 x 1080 155 in two, 212 in three (105 and 154 with chunks staged over
+// their common box and no bands); 32 x 8 masks of 3840 x 2160, 8.4 K: 622 in
+// five, 706 in eleven.  (A test that passes over voxels above or below the band
+// gains nothing: their warps wait for the others.)
 //
 // Cluster size: the one with the least time for the SM that gets most CTAs, if
 // a CTA costs 1 / S of a mask's list and 1 / 8 for its bitmask, and CTAs beside
@@ -644,6 +654,7 @@ ReprojectSplit reproject_split(int64_t n_pix, int64_t frame_cams, uint32_t list_
     r.cluster = 1;
     r.parts = r.part_threads = 0;
     r.most = UINT32_MAX;
+    r.threads = 2 * (4 * band_words(r.band_pix) + kRpStatic) <= kRpSmShared ? kRpSmThreads / 2 : kRpSmThreads;
     const int64_t masks = frame_cams * r.bands;
     sms = std::max(sms, 1);
     double best = 1e300;
@@ -657,10 +668,10 @@ ReprojectSplit reproject_split(int64_t n_pix, int64_t frame_cams, uint32_t list_
     }
     const uint32_t most = 4 * masks <= sms ? 4096u : 0u;
     if (3 * masks <= sms && list_stride > most) {
-        const int per_sm = std::min(4, 220 * 1024 / (4 * band_words(r.band_pix) + 6144));
+        const int per_sm = std::max(1, std::min(4, kRpSmShared / (4 * band_words(r.band_pix) + kRpStatic)));
         r.most = most;
         r.parts = (int)std::min<int64_t>(per_sm * (int64_t)sms / masks, ((int64_t)list_stride + 127) / 128);
-        r.part_threads = (2 * kRpThreads / per_sm) & ~31;
+        r.part_threads = (kRpSmThreads / per_sm) & ~31;
     }
     return r;
 }
@@ -686,7 +697,7 @@ cudaError_t launch_reproject(const ReprojectArgs &a, int n_frames, cudaStream_t 
     const FastDiv by_nxy = make_fast_div((uint32_t)a.nx * (uint32_t)a.ny), by_nx = make_fast_div((uint32_t)a.nx);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.n_cams * sp.bands * sp.cluster), (unsigned)n_frames);
-    cfg.blockDim = dim3(kRpThreads);
+    cfg.blockDim = dim3((unsigned)sp.threads);
     cfg.dynamicSmemBytes = (size_t)(4 * band_words(sp.band_pix));
     cfg.stream = s;
     cudaLaunchAttribute attr = {};

@@ -3,7 +3,7 @@
 // the rule without a GPU.
 //
 // input:  per call: n_pix frame_cams list_stride sms
-// output: per call: bands band_pix cluster most parts part_threads
+// output: per call: bands band_pix cluster threads most parts part_threads
 #include <cstdio>
 
 #include "psfs_internal.cuh"
@@ -18,7 +18,8 @@ int main(int argc, char **argv)
     int sms = 0;
     while (std::fscanf(f, "%lld %lld %u %d", &n_pix, &frame_cams, &stride, &sms) == 4) {
         const psfs::ReprojectSplit r = psfs::reproject_split(n_pix, frame_cams, stride, sms);
-        std::printf("%d %d %d %u %d %d\n", r.bands, r.band_pix, r.cluster, r.most, r.parts, r.part_threads);
+        std::printf("%d %d %d %d %u %d %d\n", r.bands, r.band_pix, r.cluster, r.threads, r.most, r.parts,
+                    r.part_threads);
     }
     std::fclose(f);
     return 0;

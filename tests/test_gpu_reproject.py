@@ -156,7 +156,8 @@ def test_bitmask_bands_and_clusters(width, height, n_cams, frames):
 
 
 @pytest.mark.parametrize("width,height,n_cams,frames,offset", [(67, 51, 2, 1, 0), (67, 51, 2, 3, 1), (33, 1, 1, 3, 3),
-                                                               (64, 48, 3, 2, 2), (1100, 760, 1, 1, 0)])
+                                                               (64, 48, 3, 2, 2), (1100, 760, 1, 1, 0),
+                                                               (1400, 1290, 1, 1, 1)])
 def test_parts_of_the_list(width, height, n_cams, frames, offset):
     """Few masks and lists of more than 4096 entries: parts of the list, a CTA
     each, OR-ed into a zeroed mask (masks at any byte, rows of any length, two
@@ -223,7 +224,8 @@ def _depths(grid, cam):
     return d.min(1), d.max(1)
 
 
-@pytest.mark.parametrize("width,height,frames", [(48, 40, 1), (48, 40, 320), (1100, 760, 1)])
+@pytest.mark.parametrize("width,height,frames", [(48, 40, 1), (48, 40, 320), (1100, 760, 1),
+                                                 (1400, 1290, 1)])
 def test_cubes_at_and_behind_a_camera(width, height, frames):
     """Cameras inside an 8 m grid: cubes wholly behind one, cubes at its plane
     (several of one thread, and in rounds of the list beyond its 32nd), in one
@@ -270,4 +272,21 @@ def test_cubes_behind_a_camera_cost_no_more_than_those_in_front():
         times.append(best)
     assert rec.sync() == psfs.PSFS_OK
     assert times[1] <= 10 * times[0], times
+    rec.close()
+
+
+def test_two_bands():
+    """An image of more pixels than one CTA's bitmask holds (1.77 million): two
+    bands of one mask, with one cluster per band (few frames) and one CTA (many),
+    against the oracle."""
+    width, height = 1400, 1290
+    sc = S.make_scene(seed=44, grid_n=20, cube_side=2.0, n_cams=1, width=width, height=height, focal=0.9 * width)
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+    s_ = np.random.default_rng(5).choice(sc.grid.n_voxels, 60, replace=False).astype(np.int32)
+    for frames in (1, 160):
+        lists = torch.from_numpy(s_).cuda().repeat(frames, 1)
+        counts = torch.full((frames,), s_.size, dtype=torch.int32, device="cuda")
+        got = _gpu_masks(rec, lists, counts, s_.size)
+        _check(sc.grid, sc.cams, s_.astype(np.uint32), got[0])
+        assert (got == got[0]).all()
     rec.close()
