@@ -17,7 +17,7 @@
 //
 // A cluster of S CTAs takes one particle, CTA r the cameras r, r + S, ...: 200
 // particles alone are 1.3 CTAs per SM, too few warps to cover the latency of
-// the scattered mask reads.  What the samples share is formed once per CTA in
+// the scattered mask reads (many particles: a CTA each).  What the samples share is formed once per CTA in
 // shared memory: the t and w of the sample grid, the cylinders, and n per
 // (camera, cylinder).  A warp takes 32 consecutive samples of one camera at a
 // time, so the camera's matrix comes from the constant bank and the misses
@@ -36,7 +36,6 @@ namespace psfs {
 
 namespace {
 
-constexpr int kWThreads = 512;
 constexpr int kWMaxSamples = 64;   // largest kt, kw and n_cyl
 constexpr int kWMaxCluster = 8;
 
@@ -69,28 +68,31 @@ __device__ __forceinline__ void add_to_first(int *p, int v)
     asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-__global__ void __launch_bounds__(kWThreads, 3) weights_kernel(const __grid_constant__ WeightArgs a, int S,
-                                                            FastDiv by_cyl, FastDiv by_kw)
+// kCluster false: S = 1, a particle per CTA, without cluster barriers.
+template <int kThreads, bool kCluster>
+__global__ void __launch_bounds__(kThreads, 1536 / kThreads) weights_kernel(const __grid_constant__ WeightArgs a, int S,
+                                                                            FastDiv by_cyl, FastDiv by_kw)
 {
+    constexpr int kWarps = kThreads / 32;
     __shared__ int s_miss_r[PSFS_MAX_CAMS], s_miss_e[PSFS_MAX_CAMS];   // CTA 0's are the particle's
     __shared__ float s_t[kWMaxSamples], s_w[kWMaxSamples];
     __shared__ float s_cyl[kWMaxSamples][7];                           // a, u = b - a, r
     extern __shared__ float s_n[];                                     // n: [own cameras][n_cyl][3]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int rank = (int)cluster_rank();
-    const int p = (int)blockIdx.x / S;
+    const int rank = kCluster ? (int)cluster_rank() : 0;
+    const int p = kCluster ? (int)blockIdx.x / S : (int)blockIdx.x;
     const int K = a.n_cams, W = a.W, H = a.H, n_cyl = a.n_cyl;
-    const int own = (K - rank + S - 1) / S;   // cameras rank, rank + S, ... < K
+    const int own = kCluster ? (K - rank + S - 1) / S : K;   // cameras rank, rank + S, ... < K
     if (tid < PSFS_MAX_CAMS) {
         s_miss_r[tid] = 0;
         s_miss_e[tid] = 0;
     }
     // CTA 0's counters are zero and it runs before any peer adds to them
-    cluster_arrive();
-    if (tid < a.kt) s_t[tid] = ((float)tid + 0.5f) / (float)a.kt;
-    if (tid >= 64 && tid - 64 < a.kw) s_w[tid - 64] = (2.0f * (float)(tid - 64) + 1.0f) / (float)a.kw - 1.0f;
+    if (kCluster) cluster_arrive();
+    for (int i = tid; i < a.kt; i += kThreads) s_t[i] = ((float)i + 0.5f) / (float)a.kt;
+    for (int i = kThreads - 1 - tid; i < a.kw; i += kThreads) s_w[i] = (2.0f * (float)i + 1.0f) / (float)a.kw - 1.0f;
     const float *cyl0 = a.cyl + (size_t)p * n_cyl * 7;
-    for (int it = tid; it < max(own, 1) * n_cyl; it += kWThreads) {
+    for (int it = tid; it < max(own, 1) * n_cyl; it += kThreads) {
         const int ci = it / n_cyl, q = it - ci * n_cyl;
         const int c = min(rank + ci * S, K - 1);
         const float *cy = cyl0 + q * 7;
@@ -117,19 +119,18 @@ __global__ void __launch_bounds__(kWThreads, 3) weights_kernel(const __grid_cons
         }
     }
     __syncthreads();
-    cluster_wait();
+    if (kCluster) cluster_wait();
 
     const int n_sil = a.kt * a.kw, per_cam = n_cyl * (n_sil + 2 * a.kt);
     const int blocks = (per_cam + 31) / 32;   // warp blocks of 32 samples per camera
     for (int ci = 0; ci < own; ++ci) {
-        const int c = rank + ci * S;
+        const int c = kCluster ? rank + ci * S : ci;
         const float *P = a.P[c];
         const uint8_t *m = a.masks + (size_t)c * W * H;
         const float *nrm = s_n + 3 * n_cyl * ci;
         int miss_r = 0, miss_e = 0;
         // warps start at different blocks per camera, so that the blocks left over even out
-        for (int blk = (warp + ci * (kWThreads / 32 - blocks % (kWThreads / 32))) % (kWThreads / 32); blk < blocks;
-             blk += kWThreads / 32) {
+        for (int blk = (warp + ci * (kWarps - blocks % kWarps)) % kWarps; blk < blocks; blk += kWarps) {
             const int r0 = blk * 32 + lane;
             bool miss = false, edge = false;
             if (r0 < per_cam) {
@@ -173,12 +174,21 @@ __global__ void __launch_bounds__(kWThreads, 3) weights_kernel(const __grid_cons
             miss_e += __popc(__ballot_sync(0xFFFFFFFFu, miss && edge));
         }
         if (lane == 0 && (miss_r | miss_e)) {
-            add_to_first(&s_miss_r[c], miss_r);
-            add_to_first(&s_miss_e[c], miss_e);
+            if (kCluster) {
+                add_to_first(&s_miss_r[c], miss_r);
+                add_to_first(&s_miss_e[c], miss_e);
+            } else {
+                atomicAdd(&s_miss_r[c], miss_r);
+                atomicAdd(&s_miss_e[c], miss_e);
+            }
         }
     }
-    cluster_arrive();
-    cluster_wait();
+    if (kCluster) {
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
     if (rank == 0 && tid == 0) {
         const float inv_r = 1.0f / (float)(n_cyl * a.kt * a.kw), inv_e = 1.0f / (float)(2 * n_cyl * a.kt);
         float total = 0.0f;
@@ -201,16 +211,25 @@ FastDiv make_fast_div(uint32_t d)
 
 }  // namespace
 
-// Cluster size: the largest of 1, 2, 4 and 8 whose CTAs all run at once (three
-// per SM), no more than there are cameras.
+// Cluster size: the largest of 1, 2, 4 and 8 whose CTAs of 512 threads all run
+// at once (three per SM), no more than there are cameras.  More particles take
+// a CTA each, of 512, 256 or 128 threads: no more than they have warp blocks
+// for, and fewer as long as the SMs stay full, because a CTA's set-up costs more
+// than its threads (5000 particles, one camera, 160 samples: 13 us with 128
+// threads, 17 with 256, 29 with 512, 42 with clusters of one CTA of 512; 10000,
+// eight cameras of 480: 230, 242, 275 and 312; 456, the same: 27, 19 and 19).
 cudaError_t launch_weights(const WeightArgs &a, int n_particles, cudaStream_t s)
 {
     if (n_particles <= 0) return cudaSuccess;
-    int S = 1;
-    while (S < kWMaxCluster && 2 * S <= a.n_cams && (int64_t)n_particles * 2 * S <= 3 * (int64_t)device_sm_count()) S *= 2;
+    const int64_t sms = device_sm_count();
+    int S = 1, threads = 512;
+    while (S < kWMaxCluster && 2 * S <= a.n_cams && (int64_t)n_particles * 2 * S <= 3 * sms) S *= 2;
+    const int blocks = a.n_cams * ((a.n_cyl * a.kt * (a.kw + 2) + 31) / 32);
+    while (S == 1 && threads > 128 && ((int64_t)n_particles * threads / 2 >= 1536 * sms || threads / 2 >= 32 * blocks))
+        threads /= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)n_particles * (unsigned)S);
-    cfg.blockDim = dim3(kWThreads);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = (size_t)((a.n_cams + S - 1) / S) * a.n_cyl * 3 * sizeof(float);
     cfg.stream = s;
     cudaLaunchAttribute attr = {};
@@ -219,9 +238,13 @@ cudaError_t launch_weights(const WeightArgs &a, int n_particles, cudaStream_t s)
     attr.val.clusterDim.y = 1;
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = S > 1 ? 1 : 0;
+    const auto kernel = S > 1            ? weights_kernel<512, true>
+                        : threads == 512 ? weights_kernel<512, false>
+                        : threads == 256 ? weights_kernel<256, false>
+                                         : weights_kernel<128, false>;
     const cudaError_t e =
-        cudaLaunchKernelEx(&cfg, weights_kernel, a, S, make_fast_div((uint32_t)(a.kt * a.kw + 2 * a.kt)),
+        cudaLaunchKernelEx(&cfg, kernel, a, S, make_fast_div((uint32_t)(a.kt * a.kw + 2 * a.kt)),
                            make_fast_div((uint32_t)a.kw));
     return e == cudaSuccess ? cudaGetLastError() : e;
 }

@@ -131,3 +131,48 @@ def test_clusters_and_sample_grids(n_cams, n_parts, n_cyl, kt, kw):
     keep = np.unique(np.linspace(0, n_parts - 1, 8).astype(int))
     _check(sc.cams, masks, parts[keep], w[keep], t[keep], kt, kw)
     rec.close()
+
+
+@pytest.mark.parametrize("n_cams,n_parts,n_cyl,kt,kw", [(8, 2, 10, 8, 4), (11, 5, 9, 5, 3), (32, 1, 64, 4, 2),
+                                                        (8, 200, 10, 8, 4), (3, 460, 10, 8, 4), (2, 470, 1, 2, 1),
+                                                        (3, 920, 10, 4, 2), (2, 1900, 10, 3, 2)])
+def test_clusters_of_eight_and_single_ctas(n_cams, n_parts, n_cyl, kt, kw):
+    """Eight CTAs per particle with cameras that divide among them and that do
+    not, the largest shared tables, two CTAs with several cameras each, and a
+    CTA per particle of 512, 256 and 128 threads."""
+    sc = S.make_scene(seed=54, grid_n=16, cube_side=2.2, n_cams=n_cams, width=101, height=77, focal=90.0)
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+    caps = S.body_capsules(S.random_pose(np.random.default_rng(13)), np.zeros((10, 3)))
+    masks = np.stack([(S.render_labels(c, caps) >= 0).astype(np.uint8) for c in sc.cams])
+    base = np.tile(_cyl(caps), (7, 1))[:n_cyl]
+    parts = _particles(14, n_parts, base)
+    w, t = _gpu(rec, parts, masks, kt, kw)
+    keep = np.unique(np.linspace(0, n_parts - 1, 8).astype(int))
+    _check(sc.cams, masks, parts[keep], w[keep], t[keep], kt, kw)
+    rec.close()
+
+
+def test_many_particles_of_few_samples_cost_little():
+    """5000 particles of one camera and 30 samples against 1000 of eight cameras
+    and 480: a 26th of the samples, and a third of the time here; as long a time
+    when every particle took a cluster of 512 threads."""
+    sc = S.make_scene(seed=55, grid_n=16, cube_side=2.2, n_cams=8, width=160, height=120, focal=150.0)
+    times = []
+    for n_cams, n_parts, kt, kw in ((8, 1000, 8, 4), (1, 5000, 1, 1)):
+        rec = psfs.Reconstructor(sc.grid, sc.cams[:n_cams], sc.params)
+        cyl = torch.rand((n_parts, 10, 7), device="cuda")
+        masks = torch.ones((n_cams, 120, 160), dtype=torch.uint8, device="cuda")
+        w = torch.empty(n_parts, device="cuda")
+        best = 1e9
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(10):
+                psfs.psfs_particle_weights(rec.handle, cyl, masks, w, None, kt, kw)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        times.append(best)
+        rec.close()
+    assert times[1] <= 0.7 * times[0], times
