@@ -447,3 +447,70 @@ def test_owner_list_layouts(grid_n, width, height, frames):
             assert torch.equal(many[f], one), f
         assert rec.sync() == psfs.PSFS_OK
     rec.close()
+
+
+@pytest.mark.parametrize("grid_n,n_cams,width,height", [(24, 3, 28, 20), (40, 3, 44, 32), (48, 2, 34, 33), (64, 2, 8, 6),
+                                                        (64, 1, 5, 4), (33, 1, 5, 3)])
+def test_owner_list_segments(grid_n, n_cams, width, height):
+    """Segments sorted by a lane, a warp and a CTA, in shared memory and in place,
+    in slices of every layout: 24 voxels per pixel with a last slice of 16 pixels,
+    46, about 100, thousands (beyond the buffers of a warp and of a CTA).  Whole-number sums as in test_owner_list_layouts; the batched pass, which runs
+    in the first case, gives the frames of one frame per call."""
+    frames = 5
+    sc = S.make_scene(seed=62, grid_n=grid_n, cube_side=2.0, n_cams=n_cams, width=width, height=height,
+                      focal=0.9 * width, n_frames=frames, walking=True)
+    rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+    pix = oracle.voxel_pixels(sc.grid, sc.cams)
+    bnd = oracle.reconstruct(sc.grid, sc.cams, sc.images[0], sc.mean, sc.var, sc.params)["boundary"]
+    d_occ = np.random.default_rng(8).integers(-8, 9, sc.grid.n_voxels).astype(np.float32)
+    d_occ[bnd] = 0
+    n_pix = n_cams * width * height
+    got = [torch.empty(n_pix, device="cuda") for _ in range(2)]
+    for g in got:
+        psfs.psfs_backward_slm(rec.handle, torch.full((n_pix,), 0.5, device="cuda"), to_dev(d_occ), g)
+        assert rec.sync() == psfs.PSFS_OK
+    assert torch.equal(*got)
+    pd, q = sc.params.p_detect, 0.5 * (sc.params.p_detect + sc.params.p_false_alarm)
+    want = np.concatenate([np.bincount(pix[c][pix[c] >= 0], weights=0.25 * d_occ[pix[c] >= 0].astype(np.float64),
+                                       minlength=width * height) for c in range(n_cams)])
+    want = want * ((2 * pd - 1) / 0.5 - (2 * q - 1) / 0.5)
+    np.testing.assert_allclose(got[0].cpu().numpy(), want, rtol=1e-5, atol=0)
+    batched = (n_pix * 3) % 16 == 0 and sc.grid.n_voxels % 4 == 0
+    assert batched or grid_n != 24
+    if batched:
+        rec.set_background(to_dev(sc.mean), to_dev(sc.var))
+        imgs = to_dev(sc.images)
+        occ = torch.rand((frames, sc.grid.n_voxels), generator=torch.Generator().manual_seed(1)).cuda()
+        d = torch.randn((frames, sc.grid.n_voxels), generator=torch.Generator().manual_seed(2)).cuda()
+        many, one = torch.empty((frames, n_pix), device="cuda"), torch.empty(n_pix, device="cuda")
+        psfs.psfs_backward_from_occupancy(rec.handle, frames, imgs, occ, d, many, None, None)
+        for f in range(frames):
+            psfs.psfs_backward_from_occupancy(rec.handle, 1, imgs[f], occ[f], d[f], one, None, None)
+            assert torch.equal(many[f], one), f
+        assert rec.sync() == psfs.PSFS_OK
+    rec.close()
+
+
+def test_owner_lists_of_coarse_images_build_quickly():
+    """The first adjoint call builds the owner lists: an image 64 times as coarse
+    (1450 voxels per pixel instead of 23) may not take eight times as long (a sort
+    of quadratic time took fifty times as long)."""
+    grid_n, times = 96, []
+    d_occ = torch.ones(grid_n ** 3, device="cuda")
+    for width, height in ((256, 192), (32, 24)):
+        sc = S.make_scene(seed=63, grid_n=grid_n, cube_side=2.0, n_cams=2, width=width, height=height, focal=0.9 * width)
+        n_pix = 2 * width * height
+        slm, out = torch.full((n_pix,), 0.5, device="cuda"), torch.empty(n_pix, device="cuda")
+        best = 1e9
+        for _ in range(4):
+            rec = psfs.Reconstructor(sc.grid, sc.cams, sc.params)
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            torch.cuda.synchronize()
+            a.record()
+            psfs.psfs_backward_slm(rec.handle, slm, d_occ, out)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+            rec.close()
+        times.append(best)
+    assert times[1] <= 8 * times[0], times
