@@ -2251,7 +2251,7 @@ psfs_status batch_build_frames(psfs_batch *b)
         la.zero_word = fr.count;
         la.status = b->d_words;
         e = launch_likelihood(la, b->map_dtype, false, s);
-        if (e == cudaSuccess) e = launch_fuse(fas[f], shapes[f], b->map_dtype, s);
+        if (e == cudaSuccess) e = launch_fuse(fas[f], shapes[f], b->map_dtype, s, b->frames.size() > 1);
     }
     for (int k = 0; k < kBatchStreams - 1 && e == cudaSuccess; ++k) {
         e = cudaEventRecord(b->ev_join[k], b->cap_more[k]);

@@ -29,13 +29,17 @@ namespace psfs {
 
 namespace {
 
-// FP32 maps with 16 planes per thread are held to 64 registers (8 CTAs per SM
-// instead of 6): beside other frames' kernels the occupancy is worth more than
-// the 8 bytes of spills (batches of 16 rigs 650 -> 641 us; alone 18.5 -> 18.9 us
-// a frame).  16-bit maps the other way round: 256^3 x 16 takes 114 us with
-// the compiler's own 72 registers, 124 with 64 (and 133 with more than 72).
-template <typename MapT, int LX, int WY, int TZ>
-__global__ void __launch_bounds__(32 * WY, sizeof(MapT) == 4 && TZ == 16 ? 8 : 0) fuse_kernel(const __grid_constant__ FuseArgs a, int parts_log2)
+// Beside other frames' kernels (kBeside: a batch's graph) FP32 maps with 16
+// planes per thread are held to 64 registers (8 CTAs per SM instead of 6): the
+// occupancy is then worth more than the 8 bytes of spills (batches of 16 rigs
+// 614.7 us, 619.0 without the bound; of other rigs 481 and 503).  Alone they keep
+// the compiler's own 72 (a 128^3 x 8 frame 28.9 us, 31.3 with the bound; 256^3 x
+// 16 214 and 224; 20 frames one by one beside their likelihoods 620 and 660), and
+// so do 16-bit maps (256^3 x 16: the fusion 114 us with 72, 124 with 64, 133 with
+// more than 72).
+template <typename MapT, int LX, int WY, int TZ, bool kBeside>
+__global__ void __launch_bounds__(32 * WY, kBeside && sizeof(MapT) == 4 && TZ == 16 ? 8 : 0)
+    fuse_kernel(const __grid_constant__ FuseArgs a, int parts_log2)
 {
     __shared__ int s_flags[PSFS_MAX_CAMS];
     __shared__ uint32_t s_warp_off[WY];
@@ -108,44 +112,48 @@ __global__ void __launch_bounds__(32 * WY, sizeof(MapT) == 4 && TZ == 16 ? 8 : 0
 namespace {
 
 template <typename MapT, int LX, int TZ>
-cudaError_t launch_typed(const FuseArgs &a, int parts_log2, cudaStream_t s)
+cudaError_t launch_typed(const FuseArgs &a, int parts_log2, bool beside, cudaStream_t s)
 {
-    fuse_kernel<MapT, LX, 4, TZ><<<(unsigned)a.n_tiles << parts_log2, dim3(32, 4), 0, s>>>(a, parts_log2);
+    const dim3 grid((unsigned)a.n_tiles << parts_log2), block(32, 4);
+    if (beside && sizeof(MapT) == 4 && TZ == 16)
+        fuse_kernel<MapT, LX, 4, TZ, true><<<grid, block, 0, s>>>(a, parts_log2);
+    else
+        fuse_kernel<MapT, LX, 4, TZ, false><<<grid, block, 0, s>>>(a, parts_log2);
     return cudaGetLastError();
 }
 
 template <typename MapT, int LX>
-cudaError_t launch_lx(const FuseArgs &a, int tz, cudaStream_t s)
+cudaError_t launch_lx(const FuseArgs &a, int tz, bool beside, cudaStream_t s)
 {
     const int p = tile_parts_log2(a.n_tiles, tz);
     switch (tz >> p) {
-    case 2: return launch_typed<MapT, LX, 2>(a, p, s);
-    case 4: return launch_typed<MapT, LX, 4>(a, p, s);
-    case 8: return launch_typed<MapT, LX, 8>(a, p, s);
-    case 16: return launch_typed<MapT, LX, 16>(a, p, s);
+    case 2: return launch_typed<MapT, LX, 2>(a, p, beside, s);
+    case 4: return launch_typed<MapT, LX, 4>(a, p, beside, s);
+    case 8: return launch_typed<MapT, LX, 8>(a, p, beside, s);
+    case 16: return launch_typed<MapT, LX, 16>(a, p, beside, s);
     default: return cudaErrorInvalidValue;
     }
 }
 
 template <typename MapT>
-cudaError_t launch_shape(const FuseArgs &a, const FuseShape &sh, cudaStream_t s)
+cudaError_t launch_shape(const FuseArgs &a, const FuseShape &sh, bool beside, cudaStream_t s)
 {
     if (sh.wy != 4) return cudaErrorInvalidValue;
-    if (sh.lx == 8) return launch_lx<MapT, 8>(a, sh.tz, s);
-    if (sh.lx == 16) return launch_lx<MapT, 16>(a, sh.tz, s);
-    if (sh.lx == 32) return launch_lx<MapT, 32>(a, sh.tz, s);
+    if (sh.lx == 8) return launch_lx<MapT, 8>(a, sh.tz, beside, s);
+    if (sh.lx == 16) return launch_lx<MapT, 16>(a, sh.tz, beside, s);
+    if (sh.lx == 32) return launch_lx<MapT, 32>(a, sh.tz, beside, s);
     return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-cudaError_t launch_fuse(const FuseArgs &a, const FuseShape &shape, int map_dtype, cudaStream_t s)
+cudaError_t launch_fuse(const FuseArgs &a, const FuseShape &shape, int map_dtype, cudaStream_t s, bool beside)
 {
     if (a.n_tiles <= 0) return cudaSuccess;
     if (shape.staged) return launch_fuse_staged(a, shape, map_dtype, s);
-    if (map_dtype == PSFS_MAP_F16) return launch_shape<__half>(a, shape, s);
-    if (map_dtype == PSFS_MAP_BF16) return launch_shape<__nv_bfloat16>(a, shape, s);
-    return launch_shape<float>(a, shape, s);
+    if (map_dtype == PSFS_MAP_F16) return launch_shape<__half>(a, shape, beside, s);
+    if (map_dtype == PSFS_MAP_BF16) return launch_shape<__nv_bfloat16>(a, shape, beside, s);
+    return launch_shape<float>(a, shape, beside, s);
 }
 
 }  // namespace psfs

@@ -587,7 +587,8 @@ cudaError_t launch_dl_from_occ(const float *occ, const float *d_occ, float *dl, 
                                int dl_stride, cudaStream_t s);
 cudaError_t launch_owner_pixel_group(const BackwardArgs &b, const uint32_t *off, const uint32_t *vox, int n_frames,
                                      int64_t img_fstride, bool accumulate, cudaStream_t s);
-cudaError_t launch_fuse(const FuseArgs &a, const FuseShape &shape, int map_dtype, cudaStream_t s);
+// beside: other frames' kernels run at the same time (a register bound pays).
+cudaError_t launch_fuse(const FuseArgs &a, const FuseShape &shape, int map_dtype, cudaStream_t s, bool beside = false);
 cudaError_t launch_fuse_staged(const FuseArgs &a, const FuseShape &shape, int map_dtype, cudaStream_t s);
 
 // Inner-voxel removal over the occupied-voxel lists of n frames
