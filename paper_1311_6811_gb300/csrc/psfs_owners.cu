@@ -432,35 +432,38 @@ __device__ __forceinline__ bool owner_in_grid(const BackwardArgs &b, uint32_t v)
 // slices, padded to whole groups of eight rows.  The group pass reads whole
 // 32-byte records, which no two owners share, and is faster in plain order
 // (218 against 238 us per 16 frames).
-__device__ __forceinline__ int64_t slice_of(int64_t i, uint32_t per_row)
+__device__ __forceinline__ uint32_t slice_of(uint32_t i, uint32_t per_row)
 {
-    const int64_t rows = i / (8 * (int64_t)per_row);
-    const uint32_t in = (uint32_t)(i - rows * 8 * per_row);
-    return (rows * 8 + (in & 7u)) * per_row + (in >> 3);
+    const uint32_t rows = i / (8u * per_row), in = i - rows * (8u * per_row);
+    return (rows * 8u + (in & 7u)) * per_row + (in >> 3);
 }
 
 // One frame: pixel p sums b.dl over its list in ascending voxel order, one
 // warp per slice.  Four owners' dL are in flight while the next four indices
 // load; the adds stay in ascending order.  Bound by the scattered dL reads, a
 // 32-byte sector for most owners: 59.6 us per 128^3 x 8 x 640 x 480 frame
-// (16.0 M owners), 67.8 before with each pixel's indices side by side.
+// (16.0 M owners), 67.8 before with each pixel's indices side by side.  Of few
+// owners per pixel it is the slices themselves that count: 32-bit arithmetic for
+// their order took the whole call on 96^3 voxels (2.9 per pixel) from 52.7 to
+// 50.6 us, 49.0 before there were slices.
 __global__ void __launch_bounds__(256) owner_pixel_kernel(const __grid_constant__ BackwardArgs b, const uint32_t *off,
                                                           const uint32_t *vox)
 {
-    const uint32_t per_row = max(b.f.W / 32, 1);
-    const int64_t n_slices = (b.n_pix + 31) / 32, n_padded = (n_slices + 8 * per_row - 1) / (8 * per_row) * (8 * per_row);
-    const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
-    for (int64_t i = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; i < n_padded; i += stride) {
-        const int64_t sl = slice_of(i, per_row);
+    // slices fit 32 bits: the offset scan takes at most 2^28 pixels
+    const uint32_t per_row = (uint32_t)max(b.f.W / 32, 1), n_slices = (uint32_t)((b.n_pix + 31) / 32);
+    const uint32_t n_padded = (n_slices + 8u * per_row - 1u) / (8u * per_row) * (8u * per_row);
+    const uint32_t stride = gridDim.x * (blockDim.x / 32);
+    for (uint32_t i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; i < n_padded; i += stride) {
+        const uint32_t sl = slice_of(i, per_row);
         if (sl >= n_slices) continue;
-        const int64_t p = 32 * sl + (threadIdx.x & 31);
+        const int64_t p = 32 * (int64_t)sl + (threadIdx.x & 31);
         const uint32_t e0 = __ldg(off + min(p, b.n_pix)), e1 = __ldg(off + min(p + 1, b.n_pix));
-        OwnerWalk<4> walk;
-        walk.init(vox, e0, e1);
         float acc = 0.0f;
-        uint32_t v[4];
         const uint32_t cnt = e1 - e0;
         const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, cnt);
+        OwnerWalk<4> walk;
+        walk.init(vox, e0, e1);
+        uint32_t v[4];
         walk.step(v);
         for (uint32_t j = 0; j < longest; j += 4) {
             float d[4];
