@@ -51,6 +51,19 @@ __device__ __forceinline__ bool psfs_in_bounds(bool ok, uint32_t *status)
 #define PSFS_IN_BOUNDS(cond, status) true
 #endif
 
+// What the bounds-checked build tests of the adjoint's owner lists before it
+// reads them: a pixel's segment e0 .. e1 - 1 lies in its slice's entries base ..
+// end - 1, and these in the lists (`total` entries); and an entry that a walk
+// along a slice reads lies in the slice.
+__host__ __device__ inline bool owner_segment_ok(uint32_t e0, uint32_t e1, uint32_t base, uint32_t end, uint32_t total)
+{
+    return base <= e0 && e0 <= e1 && e1 <= end && end <= total;
+}
+__host__ __device__ inline bool owner_entry_ok(const uint32_t *entry, const uint32_t *vox, uint32_t base, uint32_t end)
+{
+    return entry >= vox + base && entry < vox + end;
+}
+
 // Projection of voxel index space into one camera: (u, v, w) = M (i', j', k', 1)
 // with i' = i - (nx - 1) / 2 (likewise j', k'), rows u, v, w of 4 floats.
 struct CamMat {

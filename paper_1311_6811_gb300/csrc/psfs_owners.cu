@@ -273,14 +273,37 @@ struct OwnerWalk {
     const uint32_t *next;   // jagged: the warp's next row; otherwise the lane's next entry
     uint32_t left;          // entries of the lane not yet fetched
     bool jagged;
+#ifdef PSFS_BOUNDS_CHECK
+    const uint32_t *lists;   // and the slice's entries of them
+    uint32_t slice0, slice1;
+    uint32_t *status;
+#endif
 
-    // The slice's segment offsets: e0, e1 of this lane's pixel, the slice's ends.
-    __device__ __forceinline__ void init(const uint32_t *vox, uint32_t e0, uint32_t e1)
+    // The segment e0 .. e1 - 1 of this lane's pixel; `total` entries in all
+    // lists.  `left` is then the segment's length (0 in the bounds-checked build
+    // where it does not lie in the lists).
+    __device__ __forceinline__ void init(const uint32_t *vox, uint32_t e0, uint32_t e1, const uint32_t *total,
+                                         uint32_t *status_word)
     {
         const uint32_t base = __shfl_sync(0xFFFFFFFFu, e0, 0), end = __shfl_sync(0xFFFFFFFFu, e1, 31);
         jagged = end - base <= kSliceMax;
         next = vox + (jagged ? base : e0);
         left = e1 - e0;
+        (void)total;
+        (void)status_word;
+#ifdef PSFS_BOUNDS_CHECK
+        lists = vox;
+        slice0 = base;
+        slice1 = end;
+        status = status_word;
+        if (!PSFS_IN_BOUNDS(owner_segment_ok(e0, e1, base, end, __ldg(total)), status)) left = 0;
+#endif
+    }
+    // Whether entry q may be read.
+    __device__ __forceinline__ bool readable(const uint32_t *q) const
+    {
+        (void)q;
+        return PSFS_IN_BOUNDS(owner_entry_ok(q, lists, slice0, slice1), status);
     }
     // The next K voxels: v[k] for the first min(K, left) of them.
     __device__ __forceinline__ void step(uint32_t (&v)[K])
@@ -290,7 +313,8 @@ struct OwnerWalk {
         for (int k = 0; k < K; ++k) {
             const bool has = (uint32_t)k < left;
             const uint32_t lanes = __ballot_sync(0xFFFFFFFFu, has);
-            v[k] = has ? __ldg(next + (jagged ? __popc(lanes & lt_mask) : 0)) : 0u;
+            const uint32_t *q = next + (jagged ? __popc(lanes & lt_mask) : 0);
+            v[k] = has && readable(q) ? __ldg(q) : 0u;
             next += jagged ? __popc(lanes) : 1;
         }
         left = left > (uint32_t)K ? left - (uint32_t)K : 0u;
@@ -459,10 +483,10 @@ __global__ void __launch_bounds__(256) owner_pixel_kernel(const __grid_constant_
         const int64_t p = 32 * (int64_t)sl + (threadIdx.x & 31);
         const uint32_t e0 = __ldg(off + min(p, b.n_pix)), e1 = __ldg(off + min(p + 1, b.n_pix));
         float acc = 0.0f;
-        const uint32_t cnt = e1 - e0;
-        const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, cnt);
         OwnerWalk<4> walk;
-        walk.init(vox, e0, e1);
+        walk.init(vox, e0, e1, off + b.n_pix, b.f.status);
+        const uint32_t cnt = walk.left;
+        const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, cnt);
         uint32_t v[4];
         walk.step(v);
         for (uint32_t j = 0; j < longest; j += 4) {
@@ -539,12 +563,12 @@ __global__ void __launch_bounds__(256, 4) owner_pixel_group_kernel(const __grid_
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_lanes; p += stride) {
         const uint32_t e0 = __ldg(off + min(p, b.n_pix)), e1 = __ldg(off + min(p + 1, b.n_pix));
         OwnerWalk<K> walk;
-        walk.init(vox, e0, e1);
+        walk.init(vox, e0, e1, off + b.n_pix, b.f.status);
         float acc[kF];
 #pragma unroll
         for (int f = 0; f < kF; ++f) acc[f] = 0.0f;
         uint32_t v[K];
-        const uint32_t cnt = e1 - e0;
+        const uint32_t cnt = walk.left;
         const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, cnt);
         walk.step(v);
         for (uint32_t j = 0; j < longest; j += K) {
