@@ -32,7 +32,10 @@ namespace psfs {
 namespace {
 
 constexpr int kSX = 32, kSY = 16, kSZ = 32;   // outputs per CTA: 32 x 16 columns, at most 32 planes
-constexpr int kSCtas = 6;                      // resident per SM (40 registers)
+// resident per SM: the compiler's own 48 registers; held to 40, for six, the
+// kernel is 5 to 10 % slower (20 frames of 190^3 355 against 338 us, 9 of 93 x 110
+// x 77 27.0 against 24.9)
+constexpr int kSCtas = 5;
 constexpr int kHX = kSX + 2, kHY = kSY + 2;    // one plane with its halo: 34 x 18
 constexpr int kPlane = kHX * kHY;              // 612 floats
 constexpr int kThreads = 256;                  // 8 warps, rows y and y + 8
@@ -40,7 +43,7 @@ constexpr int kPerThread = (kPlane + kThreads - 1) / kThreads;   // 3
 constexpr int kSums = kHY * kSX;               // 576 x-sums per plane
 constexpr int kSumsPerThread = (kSums + kThreads - 1) / kThreads;   // 3
 
-__global__ void __launch_bounds__(kThreads, kSCtas) smooth_kernel(const SmoothArgs a, int tiles_z, int planes)
+__global__ void __launch_bounds__(kThreads) smooth_kernel(const SmoothArgs a, int tiles_z, int planes)
 {
     __shared__ float v[2][kPlane];
     __shared__ float sx[2][kSums];                // [kHY][kSX] x-sums per buffer
@@ -423,7 +426,7 @@ __global__ void __launch_bounds__(kTThreads, 4) smooth_tma_kernel(const __grid_c
 // the other, so a call of at most a few waves takes about waves x (planes +
 // 2) steps; the count that makes that least (32 for larger calls, where the
 // two extra planes per CTA are what counts): 9 frames of 93 x 110 x 77, 20
-// planes instead of 32, 36.4 -> 30.0 us.
+// planes instead of 32, 33.2 -> 24.9 us.
 static int best_planes(int nz, int64_t columns, int64_t slots)
 {
     int best = kSZ;
