@@ -108,7 +108,13 @@ typedef struct {
  * fusion kernel owns: a warp covers lanes_x voxels along x by 32 / lanes_x
  * along y, a CTA `warps` warps stacked along y, and each thread walks
  * voxels_z voxels along z; supported: lanes_x in {8, 16, 32}, warps = 4,
- * voxels_z in {2, 4, 8, 16} (8 or 16 when staged).  staged = 1 selects the
+ * voxels_z in {2, 4, 8, 16} (8 or 16 when staged).  Where a grid has so few
+ * tiles that the CTAs would not fill the GPU (fewer than three per SM), a
+ * direct launch for one frame, and the voxel pass of its adjoint, share a tile
+ * of 8 or 16 planes among 2 or 4 CTAs of at least 4 consecutive planes each;
+ * psfs_get_fuse_config still reports the shape that was set or tuned (so on
+ * such grids the autotuner's shapes of 8 and 16 planes may run the same
+ * kernel).  staged = 1 selects the
  * persistent kernel that copies
  * each tile's image footprint per camera into shared memory (bulk copies,
  * double-buffered) before gathering; 0 gathers from global memory.
