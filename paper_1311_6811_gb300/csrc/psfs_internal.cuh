@@ -51,6 +51,44 @@ __device__ __forceinline__ bool psfs_in_bounds(bool ok, uint32_t *status)
 #define PSFS_IN_BOUNDS(cond, status) true
 #endif
 
+// Division of 32-bit numbers by a run-time constant d.  DivAny takes any n: its
+// estimate n floor(2^32 / d) / 2^32 is at most one short.  DivSmall needs n d <
+// 2^32, where floor(n ceil(2^32 / d) / 2^32) is exact (mul = 0: d = 1).
+struct DivAny {
+    uint32_t d, mul;   // mul = floor(2^32 / d), 2^32 - 1 for d = 1
+};
+inline DivAny make_div_any(uint32_t d) { return {d, d == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d)}; }
+__device__ __forceinline__ uint32_t div_any(uint32_t n, const DivAny &f, uint32_t &rem)
+{
+    uint32_t q = __umulhi(n, f.mul);
+    rem = n - q * f.d;
+    if (rem >= f.d) {
+        ++q;
+        rem -= f.d;
+    }
+    return q;
+}
+struct DivSmall {
+    uint32_t d, mul;
+};
+inline DivSmall make_div_small(uint32_t d) { return {d, d == 1 ? 0u : (uint32_t)(((1ull << 32) + d - 1) / d)}; }
+__device__ __forceinline__ uint32_t div_small(uint32_t n, const DivSmall &f) { return f.mul ? __umulhi(n, f.mul) : n; }
+
+// This CTA's place in its cluster, and the cluster's barrier.
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync()
+{
+    cluster_arrive();
+    cluster_wait();
+}
+
 // What the bounds-checked build tests of the adjoint's owner lists before it
 // reads them: a pixel's segment e0 .. e1 - 1 lies in its slice's entries base ..
 // end - 1, and these in the lists (`total` entries); and an entry that a walk

@@ -137,25 +137,6 @@ __device__ __forceinline__ void set_bits(uint32_t *bits, int lo, int hi)
     or_word(last, last_m);
 }
 
-// Division by a run-time constant d: the estimate n floor(2^32 / d) / 2^32 is
-// at most one short.
-struct FastDiv {
-    uint32_t d, mul;   // mul = floor(2^32 / d), 2^32 - 1 for d = 1
-};
-
-__device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv &f, uint32_t &rem)
-{
-    uint32_t q = __umulhi(n, f.mul);
-    rem = n - q * f.d;
-    if (rem >= f.d) {
-        ++q;
-        rem -= f.d;
-    }
-    return q;
-}
-
-FastDiv make_fast_div(uint32_t d) { return {d, d == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d)}; }
-
 // The projection of one listed voxel's cube in camera c: the silhouette
 // polygon (n >= 3 corners, a 4-corner loop padded with its first corner, so
 // that zero-length edges cross no row), the du/dv of its edges and the
@@ -171,11 +152,11 @@ struct CubeProj {
 };
 
 // `corners`: the silhouette table as corner offsets (see kernel).
-__device__ __forceinline__ void project_cube(const ReprojectArgs &a, const float4 *corners, const FastDiv &by_nxy,
-                                             const FastDiv &by_nx, int c, uint32_t v, CubeProj &P)
+__device__ __forceinline__ void project_cube(const ReprojectArgs &a, const float4 *corners, const DivAny &by_nxy,
+                                             const DivAny &by_nx, int c, uint32_t v, CubeProj &P)
 {
     uint32_t r, ix;
-    const uint32_t kz = fast_div(v, by_nxy, r), jy = fast_div(r, by_nx, ix);
+    const uint32_t kz = div_any(v, by_nxy, r), jy = div_any(r, by_nx, ix);
     const int W = a.W, H = a.H;
     float m[12];
 #pragma unroll
@@ -320,8 +301,8 @@ __device__ void slab_test_pixels(const ReprojectArgs &a, int c, const CubeProj &
 // pixels are all set passed over.  A cube at the camera plane may cover the
 // whole image: 3000 voxels around a camera at 320 x 240 take 0.37 ms, 5.4 with
 // one thread per cube.
-__device__ __forceinline__ void slab_test_queue(const ReprojectArgs &a, const float4 *corners, const FastDiv by_nxy,
-                                             const FastDiv by_nx, int c, const uint32_t *queue, uint32_t n,
+__device__ __forceinline__ void slab_test_queue(const ReprojectArgs &a, const float4 *corners, const DivAny by_nxy,
+                                             const DivAny by_nx, int c, const uint32_t *queue, uint32_t n,
                                              uint32_t *bits, int p0, int p1)
 {
     const int lane = threadIdx.x & 31, W = a.W;
@@ -348,18 +329,6 @@ __device__ __forceinline__ void slab_test_queue(const ReprojectArgs &a, const fl
 }
 
 // ---- the cluster's other bitmasks (distributed shared memory) ----
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-
 __device__ __forceinline__ uint32_t load_peer(const uint32_t *p, uint32_t rank)
 {
     uint32_t a, v;
@@ -462,8 +431,8 @@ __device__ __forceinline__ RpPlace locate(const ReprojectArgs &a, int bands, int
 
 // The slab tests of the voxels that the threads of a CTA left pending (bit i:
 // mine[i * step]), one of each thread at a time.
-__device__ __forceinline__ void slab_phase(const ReprojectArgs &a, const float4 *corners, const FastDiv by_nxy,
-                                        const FastDiv by_nx, int c, const uint32_t *mine, uint64_t step,
+__device__ __forceinline__ void slab_phase(const ReprojectArgs &a, const float4 *corners, const DivAny by_nxy,
+                                        const DivAny by_nx, int c, const uint32_t *mine, uint64_t step,
                                         uint32_t pending, uint32_t *bits, int p0, int p1)
 {
     __shared__ uint32_t queue[kRpSmThreads], queued;
@@ -494,11 +463,11 @@ __device__ __forceinline__ void slab_phase(const ReprojectArgs &a, const float4 
 // voxels staged as bytes over their common box, OR-ed into a zeroed mask word
 // by word): 275 us; with eight corner depths, corner offsets from selects and
 // integer divisions per voxel instead of the depth bound, the offset table and
-// fast_div: 175 us; with a loop over the words of each run in set_bits: 164 us.
+// div_any: 175 us; with a loop over the words of each run in set_bits: 164 us.
 template <bool kParts>
 __global__ void __launch_bounds__(kRpSmThreads, 1) reproject_kernel(const __grid_constant__ ReprojectArgs a,
                                                                   const __grid_constant__ SilTable sil,
-                                                                  FastDiv by_nxy, FastDiv by_nx, int bands,
+                                                                  DivAny by_nxy, DivAny by_nx, int bands,
                                                                   int band_pix, int n, uint32_t most)
 {
     extern __shared__ __align__(16) uint32_t bits[];   // band_words(band_pix) words, the last of them zero
@@ -694,7 +663,7 @@ cudaError_t launch_reproject(const ReprojectArgs &a, int n_frames, cudaStream_t 
         }
         configured[dev] = true;
     }
-    const FastDiv by_nxy = make_fast_div((uint32_t)a.nx * (uint32_t)a.ny), by_nx = make_fast_div((uint32_t)a.nx);
+    const DivAny by_nxy = make_div_any((uint32_t)a.nx * (uint32_t)a.ny), by_nx = make_div_any((uint32_t)a.nx);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.n_cams * sp.bands * sp.cluster), (unsigned)n_frames);
     cfg.blockDim = dim3((unsigned)sp.threads);

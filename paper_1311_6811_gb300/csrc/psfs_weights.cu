@@ -39,26 +39,7 @@ namespace {
 constexpr int kWMaxSamples = 64;   // largest kt, kw and n_cyl
 constexpr int kWMaxCluster = 8;
 
-// Division by a run-time constant d: q = floor(n ceil(2^32 / d) / 2^32),
-// exact for n d < 2^32 (d = 1 is handled by the caller's ceil(2^32 / 1) not
-// fitting 32 bits: mul = 0 means "divide by one").
-struct FastDiv {
-    uint32_t d, mul;
-};
-
-__device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv &f) { return f.mul ? __umulhi(n, f.mul) : n; }
-
 __device__ __forceinline__ bool mask_at(const uint8_t *m, int W, int x, int y) { return __ldg(m + (size_t)y * W + x) != 0; }
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 
 // *p += v in the shared memory of the cluster's CTA 0.
 __device__ __forceinline__ void add_to_first(int *p, int v)
@@ -71,7 +52,7 @@ __device__ __forceinline__ void add_to_first(int *p, int v)
 // kCluster false: S = 1, a particle per CTA, without cluster barriers.
 template <int kThreads, bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1536 / kThreads) weights_kernel(const __grid_constant__ WeightArgs a, int S,
-                                                                            FastDiv by_cyl, FastDiv by_kw)
+                                                                            DivSmall by_cyl, DivSmall by_kw)
 {
     constexpr int kWarps = kThreads / 32;
     __shared__ int s_miss_r[PSFS_MAX_CAMS], s_miss_e[PSFS_MAX_CAMS];   // CTA 0's are the particle's
@@ -134,10 +115,10 @@ __global__ void __launch_bounds__(kThreads, 1536 / kThreads) weights_kernel(cons
             const int r0 = blk * 32 + lane;
             bool miss = false, edge = false;
             if (r0 < per_cam) {
-                const int q = (int)fast_div((uint32_t)r0, by_cyl), smp = r0 - q * (int)by_cyl.d;
+                const int q = (int)div_small((uint32_t)r0, by_cyl), smp = r0 - q * (int)by_cyl.d;
                 float t, w;
                 if (smp < n_sil) {   // silhouette sample (k, l)
-                    const int k = (int)fast_div((uint32_t)smp, by_kw), l = smp - k * a.kw;
+                    const int k = (int)div_small((uint32_t)smp, by_kw), l = smp - k * a.kw;
                     t = s_t[k];
                     w = s_w[l];
                 } else {             // edge sample (k, side)
@@ -183,12 +164,10 @@ __global__ void __launch_bounds__(kThreads, 1536 / kThreads) weights_kernel(cons
             }
         }
     }
-    if (kCluster) {
-        cluster_arrive();
-        cluster_wait();
-    } else {
+    if (kCluster)
+        cluster_sync();
+    else
         __syncthreads();
-    }
     if (rank == 0 && tid == 0) {
         const float inv_r = 1.0f / (float)(n_cyl * a.kt * a.kw), inv_e = 1.0f / (float)(2 * n_cyl * a.kt);
         float total = 0.0f;
@@ -202,11 +181,6 @@ __global__ void __launch_bounds__(kThreads, 1536 / kThreads) weights_kernel(cons
         }
         a.weights[p] = expf(-total);
     }
-}
-
-FastDiv make_fast_div(uint32_t d)
-{
-    return {d, d == 1 ? 0u : (uint32_t)(((1ull << 32) + d - 1) / d)};
 }
 
 }  // namespace
@@ -244,8 +218,8 @@ cudaError_t launch_weights(const WeightArgs &a, int n_particles, cudaStream_t s)
                         : threads == 256 ? weights_kernel<256, false>
                                          : weights_kernel<128, false>;
     const cudaError_t e =
-        cudaLaunchKernelEx(&cfg, kernel, a, S, make_fast_div((uint32_t)(a.kt * a.kw + 2 * a.kt)),
-                           make_fast_div((uint32_t)a.kw));
+        cudaLaunchKernelEx(&cfg, kernel, a, S, make_div_small((uint32_t)(a.kt * a.kw + 2 * a.kt)),
+                           make_div_small((uint32_t)a.kw));
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
