@@ -40,8 +40,9 @@ struct TileCoords {
 // Parts that the tiles of a plan are cut into along z, a CTA each (log2): a
 // grid of few tiles would leave most of the GPU idle while each thread walks
 // its whole column of voxels.  Cut until there are three CTAs per SM or four
-// planes per part; a tile's camera flags hold for its parts.  64^3 x 4
-// cameras, 128 tiles of 16 planes: fusion 10.2 -> 8.1 us
+// planes per part; a tile's camera flags hold for its parts.  64^3 x 4 cameras,
+// 128 tiles of 16 planes: the adjoint's voxel pass 14.3 -> 8.2 us, a batch of 16
+// such rigs 78 -> 67 (one frame per call is bound by its launches either way).
 inline int tile_parts_log2(int n_tiles, int tz)
 {
     int s = 0;

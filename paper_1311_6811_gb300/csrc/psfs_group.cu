@@ -151,8 +151,9 @@ struct GLayout {
 
 // Two frames of one pixel at once: pixel_quad and log_ratio_of_r with every
 // multiply, add and fma on both frames in one packed instruction (the same
-// operations on each, so the same bits).  The likelihood is bound by issue,
-// and beside a fusion it takes the issue slots that one lacks: 100-frame
+// operations on each, so the same bits).  Alone the likelihood takes 70 % of
+// DRAM's peak and 49 % of the issue slots (16 FP32 frames, ncu); beside a
+// fusion, which waits for its gathers, issue slots are what they share: 100-frame
 // sequence of 128^3 x 8 1095 -> 1064 us, 64 frames with 16-bit maps 544 -> 496.
 __device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
 

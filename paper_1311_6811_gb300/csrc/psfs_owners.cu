@@ -464,8 +464,9 @@ __device__ __forceinline__ uint32_t slice_of(uint32_t i, uint32_t per_row)
 
 // One frame: pixel p sums b.dl over its list in ascending voxel order, one
 // warp per slice.  Four owners' dL are in flight while the next four indices
-// load; the adds stay in ascending order.  Bound by the scattered dL reads, a
-// 32-byte sector for most owners: 59.6 us per 128^3 x 8 x 640 x 480 frame
+// load; the adds stay in ascending order.  Its warps wait for the scattered dL
+// reads, a 32-byte sector for most owners (ncu: long scoreboard; L1 59 %, issue
+// 55 %, DRAM 40 %, 79 % of the warps active): 59.6 us per 128^3 x 8 x 640 x 480 frame
 // (16.0 M owners), 67.8 before with each pixel's indices side by side.  Of few
 // owners per pixel it is the slices themselves that count: 32-bit arithmetic for
 // their order took the whole call on 96^3 voxels (2.9 per pixel) from 52.7 to
@@ -547,8 +548,8 @@ __device__ __forceinline__ void load_record(const float *rec, bool on, uint32_t 
 // d_slm (frame f at b.d_slm + f n_pix) is bit-identical to one frame per
 // call; d_mean and d_var receive the frames' gradients added in frame order
 // to 0 (or, with `accumulate`, to what they hold).
-// Bound by the record reads (1.0 GB of sectors per 16 frames of 128^3 x 8):
-// 218 us per 16 frames; 305 when each frame's colours were byte loads in that
+// Issue slots (66 %) and the record reads (1.0 GB of sectors per 16 frames of
+// 128^3 x 8; L2 48 %, 45 % of the warps active) hold it: 214-218 us per 16 frames; 305 when each frame's colours were byte loads in that
 // frame's branch, a memory latency each.  Four CTAs per SM: 64 registers.
 template <int R>
 __global__ void __launch_bounds__(256, 4) owner_pixel_group_kernel(const __grid_constant__ BackwardArgs b,

@@ -242,10 +242,13 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *tmap, 
 // looks for them (ballots into s_bal) in the planes whose largest value is
 // above it, and the compaction (one atomicAdd per warp) visits these planes.
 //
-// Bound by DRAM: 100 frames of 128^3 (8.4 MB in, 8.4 MB out each) take 310 us
-// with the list, 5.4 TB/s, 80 % of the copy rate.  Before (one row of four
-// columns per thread, three rows of x-sums per output row, a CTA barrier per
-// plane, every plane's ballots kept and walked again): 479 us, issue-bound.
+// 100 frames of 128^3 (8.4 MB in, 8.4 MB out each) take 312 us with the list,
+// 5.4 TB/s, 79 % of the copy rate.  Fewer frames reach less of it: 32 (1024 CTAs,
+// 1.7 waves of the 608 that are resident) 3.9 TB/s, DRAM at 46 %, 28 % of the issue
+// slots and 22 % of the warps active (ncu): the last wave, and the loads that each
+// thread waits for.  Before (one row of four columns per thread, three rows of
+// x-sums per output row, a CTA barrier per plane, every plane's ballots kept and
+// walked again): 479 us, 82 % of the issue slots.
 __global__ void __launch_bounds__(kTThreads, 4) smooth_tma_kernel(const __grid_constant__ SmoothArgs a, int tiles_x,
                                                                   int tiles_y, int tz)
 {
