@@ -744,7 +744,7 @@ def run_ours(args):
                 "alg_bytes_per_launch": stages[dom]["alg_bytes_per_launch"],
                 "units_per_step": units,
                 "note": ("the fusion kernels are bound by the L2 -> L1 sector rate of their gathers (one 32-byte "
-                         "sector per voxel, camera and 8 FP32 frames; ncu: L2 62 %, L1 77 % busy), not by HBM; "
+                         "sector per voxel, camera and 8 FP32 frames; ncu: L2 59 %, L1 89 % busy), not by HBM; "
                          "roofline_sequence gives the whole step against HBM")
                         if dom == "fuse" else None}
     # the whole step against the bytes the grouped method moves: per unit of
@@ -831,7 +831,7 @@ def run_ours(args):
                             "alg_bytes_per_frame": rp_bytes,
                             "achieved_gbs": rp_bytes / (us_rp * 1e-6) / 1e9,
                             "hbm_frac": rp_bytes / (us_rp * 1e-6) / 1e9 / peak_s,
-                            "note": "psfs_reproject of the step's surface lists in one call (1 kernel): silhouette polygons "
+                            "note": "psfs_reproject of the step's surface lists in one call (1 kernel, a second one for few masks): silhouette polygons "
                                     "of the listed cubes set in a shared-memory bitmask per camera, written once"}
         # tracker weights of 200 particles (10 cylinders each, around frame 0's
         # body) against frame 0's silhouettes

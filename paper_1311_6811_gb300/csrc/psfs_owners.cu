@@ -549,8 +549,9 @@ __device__ __forceinline__ void load_record(const float *rec, bool on, uint32_t 
 // call; d_mean and d_var receive the frames' gradients added in frame order
 // to 0 (or, with `accumulate`, to what they hold).
 // Issue slots (66 %) and the record reads (1.0 GB of sectors per 16 frames of
-// 128^3 x 8; L2 48 %, 45 % of the warps active) hold it: 214-218 us per 16 frames; 305 when each frame's colours were byte loads in that
-// frame's branch, a memory latency each.  Four CTAs per SM: 64 registers.
+// 128^3 x 8; L2 48 %, 45 % of the warps active) hold it: 214-218 us per 16 frames;
+// 305 when each frame's colours were byte loads in that frame's branch, a memory
+// latency each.  Four CTAs per SM: 64 registers.
 template <int R>
 __global__ void __launch_bounds__(256, 4) owner_pixel_group_kernel(const __grid_constant__ BackwardArgs b,
                                                                 const uint32_t *off, const uint32_t *vox,
